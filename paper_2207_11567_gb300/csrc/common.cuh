@@ -195,8 +195,23 @@ constexpr int LB_BLOCK = 128;
 // link word bit 30: the cell has interpolated bounce-back links (it is on the wall list)
 constexpr uint32_t LINK_WALL = 1u << 30;
 
+// Quotient of a 31-bit unsigned number by a divisor known at launch: one high product, one add,
+// one shift (multiplier 2^32 (2^s - d) / d + 1 with s = ceil(log2 d)).
+struct FastDiv {
+  uint32_t mul = 1, shift = 0;
+  FastDiv() = default;
+  explicit FastDiv(uint32_t d) {
+    while ((1ull << shift) < d) ++shift;
+    mul = (uint32_t)(((1ull << 32) * ((1ull << shift) - d)) / d + 1);
+  }
+  __device__ __forceinline__ int div(int n) const {
+    return (int)((__umulhi((uint32_t)n, mul) + (uint32_t)n) >> shift);
+  }
+};
+
 template <typename R> struct LBArgs {
   Geo geo;
+  FastDiv div_nx, div_ny;  // lb_pair_kernel: cell index to (x, y, z)
   const void* g_in;
   void* g_out;
   const uint32_t* links;

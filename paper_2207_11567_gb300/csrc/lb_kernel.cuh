@@ -1,5 +1,5 @@
-// Fused pull-stream + collide kernel of the pressure/momentum lattice Boltzmann solver
-// (Section 2.1-2.2), one thread per cell, lattice units (c_s^2 = 1/3).
+// Fused pull-stream + collide kernels of the pressure/momentum lattice Boltzmann solver
+// (Section 2.1-2.2), one or two cells per thread, lattice units (c_s^2 = 1/3).
 //
 // Per fluid cell:
 //   stream   g_i(r) = g*_i(r - c_i) (Eq. 1, pull), bounce-back g_i = g*_{Q-1-i}(r) on links
@@ -19,7 +19,7 @@
 // g*_i / w_i - P_ref = rho/3 (h*_i / w_i - 1) + S + xi_i / 2; the cumulant collision works on
 // h - h_eq with h_eq the product-form equilibrium, whose central moments are known exactly.
 #pragma once
-#include "common.cuh"
+#include "packed.cuh"
 
 namespace hlbm {
 
@@ -174,6 +174,605 @@ __device__ __forceinline__ void add_delta_eq(R* m, const R* dx, const R* dy, con
   }
 }
 
+// ------------------------------------------------------------------ collision, full relaxation
+// Cumulant collision with full relaxation of the orders 3..6 (the default rates), Eq. 2, 7, 13 and
+// 9-12 of one cell, for V = float, double or F2 (two cells): q[] comes in as the pulled populations
+// q_i = g_i / w_i - P_ref and goes out as the new stored ones. It works on sums over the lattice
+// instead of per-population terms, one axis at a time:
+// * The ten raw moments M_0, M_a, M_ab = 6^D sum_i w_i q_i (1, c_a, c_a c_b): per line of three
+//   (1/6, 2/3, 1/6)(q_-, q_0, q_+) the sums q_- + 4 q_0 + q_+, q_+ - q_-, q_+ + q_-, so that no
+//   weight is multiplied in.
+// * u_a = M_a / (2^D m), m = rho 3^(D-1): the reciprocal and one residual correction, which
+//   keeps the momentum of the stored populations (they are rebuilt from u with the same m) free of
+//   a rounding that would repeat every step. With G = u . grad rho and L = rho cs2 Lambda, the
+//   closed forms of the source's moments (k_0 = L + G/3, k_ab = L u_a u_b + (g_a u_b + g_b u_a)/9
+//   [+ L/3 + G/9 for a = b]) leave for the second central moments of h - h_eq
+//     n_ab = (3/rho) (A_ab - delta_ab A_0 / 3) - u_a u_b (1 + G / (2 rho)) + (g_a u_b + g_b u_a)/(6 rho)
+//   (A = M / 6^D; L cancels).
+// * Relaxed to s_ab (deviator at 1/tau, trace at omega_b), the populations h* have unit mass,
+//   velocity u, covariance 1/3 + s_ab and no cumulants beyond: their raw moments follow from
+//   Isserlis' theorem, written as deviations from those of the rest weights so that every quantity
+//   is small.
+// * Back to populations one axis at a time, (m_2 - m_1, m_0 - m_2, m_2 + m_1); the factors 1/2 of
+//   that inverse, 1 / w_i and rho / 3 together are m / 2^(number of zero components of c_i).
+// * The half source xi_i / 2 of Eq. 8 is, along x, a polynomial of degree 2 in c_x (c_x^3 = c_x)
+//   whose coefficients are formed once per line and added there.
+// About 480 operations per cell of D3Q27, against about 1080 with the transforms of all 27 central
+// moments and per-population source terms. Taken by isothermal and 2-D runs from lb_pair_kernel and by
+// FP64 (planar flame 256x8: stream-collide 22.8 -> 16.5 us); error of u after 20 steps of the cold swirl
+// against 64-bit values 2.4e-7 before, 1.5e-7 with it.
+template <int D, typename V, bool THERMAL> struct LBCell {
+  V rho, lam;           // density, Lambda (with the thermodynamic-pressure term)
+  V gx, gy, gz;         // density gradient
+  V u[3], usq;          // out: velocity, its square
+  V psum, rl3;          // out: sum of g - P_ref, rho cs2 Lambda
+};
+
+template <int D, typename V, bool THERMAL, typename R>
+__device__ __forceinline__ void collide_full(V* q, LBCell<D, V, THERMAL>& c, const V nu3, const LBArgs<R>& a) {
+  constexpr int Q = Lat<D>::Q;
+  const V one = splat<V>(1.0), two = splat<V>(2.0), four = splat<V>(4.0), half = splat<V>(0.5);
+  const V third = splat<V>(1.0 / 3.0), zero = splat<V>(0.0);
+  // raw moments: x lines, then y, then z; slot a + 3 b (+ 9 c) of m[]
+#pragma unroll
+  for (int j = 0; j < Q / 3; ++j) {
+    const V s = q[3 * j] + q[3 * j + 2], d = q[3 * j + 2] - q[3 * j];
+    q[3 * j] = fma_(four, q[3 * j + 1], s);
+    q[3 * j + 1] = d;
+    q[3 * j + 2] = s;
+  }
+#pragma unroll
+  for (int k = 0; k < Q / 9; ++k) {
+    V* p = q + 9 * k;
+    {
+      const V s = p[0] + p[6], d = p[6] - p[0];
+      p[0] = fma_(four, p[3], s);
+      p[3] = d;
+      p[6] = s;
+    }
+    {
+      const V s = p[1] + p[7], d = p[7] - p[1];
+      p[1] = fma_(four, p[4], s);
+      p[4] = d;
+    }
+    p[2] = fma_(four, p[5], p[2] + p[8]);
+  }
+  V M0, M[3], Md[3], Mo[3];  // Md: xx, yy, zz; Mo: xy, xz, yz
+  if constexpr (D == 3) {
+    const V s0 = q[0] + q[18];
+    M0 = fma_(four, q[9], s0);
+    M[2] = q[18] - q[0];
+    Md[2] = s0;
+    M[0] = fma_(four, q[10], q[1] + q[19]);
+    Mo[1] = q[19] - q[1];
+    M[1] = fma_(four, q[12], q[3] + q[21]);
+    Mo[2] = q[21] - q[3];
+    Md[0] = fma_(four, q[11], q[2] + q[20]);
+    Md[1] = fma_(four, q[15], q[6] + q[24]);
+    Mo[0] = fma_(four, q[13], q[4] + q[22]);
+  } else {
+    M0 = q[0];
+    M[0] = q[1];
+    M[1] = q[3];
+    M[2] = Md[2] = Mo[1] = Mo[2] = zero;
+    Md[0] = q[2];
+    Md[1] = q[6];
+    Mo[0] = q[4];
+  }
+  // velocity and pressure
+  const V mm = splat<V>(D == 3 ? 9.0 : 3.0) * c.rho, m4 = splat<V>(D == 3 ? 8.0 : 4.0) * mm;
+  const V im4 = rcp_(m4);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const V t = M[d] * im4;
+    c.u[d] = fma_(fma_(zero - m4, t, M[d]), im4, t);
+  }
+  if constexpr (D == 2) c.u[2] = zero;
+  const V ux = c.u[0], uy = c.u[1], uz = c.u[2];
+  const V uxx = ux * ux, uyy = uy * uy, uzz = D == 3 ? uz * uz : zero;
+  c.usq = D == 3 ? uxx + uyy + uzz : uxx + uyy;
+  // 6^-D in two parts: the sum must not lose or gain a fixed fraction each step
+  constexpr double sc = D == 3 ? 1.0 / 216.0 : 1.0 / 36.0;
+  const V sc_hi = splat<V>(sc);
+  c.psum = sizeof(R) == 4 ? fma_(M0, splat<V>(sc - (double)(float)sc), M0 * sc_hi) : M0 * sc_hi;
+  V S = c.psum;
+  c.rl3 = zero;
+  V G = zero, hL = zero, c1 = one, c2 = zero;
+  if constexpr (THERMAL) {
+    c.rl3 = c.rho * c.lam * third;
+    G = fma_(ux, c.gx, uy * c.gy);
+    if constexpr (D == 3) G = fma_(uz, c.gz, G);
+    hL = half * c.rl3;
+    S = fma_(splat<V>(1.0 / 6.0), G, S + hL);
+    c2 = splat<V>(D == 3 ? 12.0 : 2.0) * im4;  // 1 / (6 rho)
+    c1 = fma_(splat<V>(3.0) * c2, G, one);     // 1 + G / (2 rho)
+  }
+  // second central moments of h - h_eq. (3/rho) / 6^D = im4 (D3Q27: 3 / (216 rho) = 1 / (72 rho);
+  // D2Q9: 3 / (36 rho) = 1 / (12 rho))
+  const V M0t = M0 * third;
+  V nd[3], no[3];  // xx, yy, zz; xy, xz, yz
+  {
+    const V vx = c1 * ux, vy = c1 * uy, vz = c1 * uz;
+    V b[3] = {ux * vx, uy * vy, uz * vz}, bo[3] = {ux * vy, ux * vz, uy * vz};
+    if constexpr (THERMAL) {
+      const V hx = c2 * c.gx, hy = c2 * c.gy, hz = c2 * c.gz;
+      const V tx = two * hx, ty = two * hy, tz = two * hz;
+      b[0] = b[0] - tx * ux;
+      b[1] = b[1] - ty * uy;
+      bo[0] = bo[0] - fma_(hx, uy, hy * ux);
+      if constexpr (D == 3) {
+        b[2] = b[2] - tz * uz;
+        bo[1] = bo[1] - fma_(hx, uz, hz * ux);
+        bo[2] = bo[2] - fma_(hy, uz, hz * uy);
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d) nd[d] = fma_(im4, Md[d] - M0t, zero - b[d]);
+    if constexpr (D == 2) nd[2] = zero;
+    no[0] = fma_(im4, Mo[0], zero - bo[0]);
+    no[1] = D == 3 ? fma_(im4, Mo[1], zero - bo[1]) : zero;
+    no[2] = D == 3 ? fma_(im4, Mo[2], zero - bo[2]) : zero;
+  }
+  const V tr = (D == 3 ? third : half) * (D == 3 ? nd[0] + nd[1] + nd[2] : nd[0] + nd[1]);
+#pragma unroll
+  for (int d = 0; d < D; ++d) nd[d] = nd[d] - tr;
+  // relaxation time (Eq. 12) with the Smagorinsky closure on the deviator
+  const V inv_rho = splat<V>(D == 3 ? 72.0 : 12.0) * im4;
+  const V tau0 = THERMAL ? fma_(nu3, inv_rho, half) : nu3 + half;
+  V tau = tau0;
+  if (a.smag_k > R(0)) {
+    V n2 = fma_(nd[0], nd[0], nd[1] * nd[1]), o2 = no[0] * no[0];
+    if constexpr (D == 3) {
+      n2 = fma_(nd[2], nd[2], n2);
+      o2 = fma_(no[1], no[1], fma_(no[2], no[2], o2));
+    }
+    n2 = fma_(two, o2, n2);
+    tau = half * (tau0 + sqrt_pos(fma_(tau0, tau0, splat<V>(a.smag_k) * sqrt_approx(n2))));
+  }
+  const V o1 = one - rcp_(tau);
+  const V obt = splat<V>(R(1) - a.omega_b) * tr;
+  // relaxed covariance deviations s and raw second moments P = s + u u, T = 1/3 + P
+  const V sxx = fma_(o1, nd[0], obt), syy = fma_(o1, nd[1], obt), sxy = o1 * no[0];
+  const V Pxx = sxx + uxx, Pyy = syy + uyy, uxy = ux * uy, Pxy = sxy + uxy;
+  const V Txx = third + Pxx, Tyy = third + Pyy;
+  const V ux2 = two * ux, uy2 = two * uy;
+  // raw moments of h* minus those of the rest weights, slots a + 3 b + 9 c
+  q[1] = ux; q[3] = uy; q[2] = Pxx; q[6] = Pyy; q[4] = Pxy;
+  q[5] = fma_(uy, Txx, ux2 * sxy);
+  q[7] = fma_(ux, Tyy, uy2 * sxy);
+  q[8] = fma_(two * sxy, fma_(two, Pxy, zero - sxy), fma_(Txx, Pyy, third * Pxx));
+  if constexpr (D == 3) {
+    const V szz = fma_(o1, nd[2], obt), sxz = o1 * no[1], syz = o1 * no[2];
+    const V Pzz = szz + uzz, uxz = ux * uz, uyz = uy * uz, Pxz = sxz + uxz, Pyz = syz + uyz;
+    const V Tzz = third + Pzz, uz2 = two * uz;
+    const V sxy2 = two * sxy, sxz2 = two * sxz, syz2 = two * syz;
+    q[9] = uz; q[18] = Pzz; q[10] = Pxz; q[12] = Pyz;
+    q[11] = fma_(uz, Txx, ux2 * sxz);  // xxz
+    q[15] = fma_(uz, Tyy, uy2 * syz);  // yyz
+    q[19] = fma_(ux, Tzz, uz2 * sxz);  // xzz
+    q[21] = fma_(uy, Tzz, uz2 * syz);  // yzz
+    q[13] = fma_(ux, Pyz, fma_(uy, sxz, uz * sxy));  // xyz
+    q[20] = fma_(sxz2, fma_(two, Pxz, zero - sxz), fma_(Txx, Pzz, third * Pxx));  // xxzz
+    q[24] = fma_(syz2, fma_(two, Pyz, zero - syz), fma_(Tyy, Pzz, third * Pyy));  // yyzz
+    q[14] = fma_(sxz2, Pxy, fma_(sxy2, uxz, Txx * Pyz));  // xxyz
+    q[16] = fma_(syz2, Pxy, fma_(sxy2, uyz, Tyy * Pxz));  // xyyz
+    q[22] = fma_(syz2, Pxz, fma_(sxz2, uyz, Tzz * Pxy));  // xyzz
+    const V ninth = splat<V>(1.0 / 9.0);
+    q[17] = fma_(uz, ninth + q[8], fma_(sxz2, q[7], syz2 * q[5]));    // xxyyz
+    q[23] = fma_(uy, ninth + q[20], fma_(sxy2, q[19], syz2 * q[11]));  // xxyzz
+    q[25] = fma_(ux, ninth + q[24], fma_(sxy2, q[21], sxz2 * q[15]));  // xyyzz
+    q[26] = fma_(uz, q[17], fma_(sxz2, q[16], fma_(syz2, q[14], fma_(ninth, szz, (third + szz) * q[8]))));
+    // back along z: slots of equal (a, b); the mass moment is zero
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      const V m1 = q[j + 9], m2 = q[j + 18];
+      q[j + 9] = j == 0 ? zero - m2 : q[j] - m2;
+      q[j] = m2 - m1;
+      q[j + 18] = m2 + m1;
+    }
+  }
+  // back along y
+#pragma unroll
+  for (int k = 0; k < Q / 9; ++k)
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      V* p = q + 9 * k + x;
+      const V m1 = p[3], m2 = p[6];
+      const bool mass = D == 2 && x == 0;
+      p[3] = mass ? zero - m2 : p[0] - m2;
+      p[0] = m2 - m1;
+      p[6] = m2 + m1;
+    }
+  // back along x, with the scale to stored populations, S and the half source
+  V fac[D + 1];  // by number of nonzero components
+  fac[D] = mm;
+#pragma unroll
+  for (int k = D - 1; k >= 0; --k) fac[k] = half * fac[k + 1];
+  V hgx = zero, hgy = zero, hgz = zero, hG = zero, e2 = zero, eb = zero;
+  if constexpr (THERMAL) {
+    hgx = half * c.gx;
+    hgy = half * c.gy;
+    hgz = half * c.gz;
+    hG = half * G;
+    e2 = splat<V>(1.5) * uxx;
+    eb = splat<V>(-0.5) * c.usq;
+    S = S + hL;
+  }
+#pragma unroll
+  for (int j = 0; j < Q / 3; ++j) {
+    const int jy = j % 3 - 1, jz = D == 3 ? j / 3 - 1 : 0;
+    const int k = (jy != 0) + (jz != 0);
+    const V m0 = q[3 * j], m1 = q[3 * j + 1], m2 = q[3 * j + 2];
+    V p0 = S, p1 = zero, p02 = S;
+    if constexpr (THERMAL) {
+      // xi / 2 = e (c . g - G) / 2 with e = e0 + e1 c_x + e2 c_x^2 and c . g - G = b + g_x c_x
+      V e0 = eb, e1 = ux, b = zero - hG;
+      if (k) {
+        const V ay = jy > 0 ? uy : zero - uy, az = jz > 0 ? uz : zero - uz;
+        const V au = jy ? (jz ? (jz > 0 ? ay + uz : ay - uz) : ay) : az;
+        e0 = fma_(au, fma_(splat<V>(1.5), au, one), eb);
+        e1 = ux * fma_(splat<V>(3.0), au, one);
+        if (jy) b = jy > 0 ? b + hgy : b - hgy;
+        if (jz) b = jz > 0 ? b + hgz : b - hgz;
+      }
+      p0 = fma_(e0, b, S);
+      p1 = fma_(e0 + e2, hgx, e1 * b);
+      p02 = fma_(e1, hgx, fma_(e2, b, p0));
+    }
+    const V A = fma_(fac[k + 1], m2, p02);
+    const V B = THERMAL ? fma_(fac[k + 1], m1, p1) : fac[k + 1] * m1;
+    q[3 * j] = A - B;
+    q[3 * j + 1] = fma_(fac[k], m0 - m2, p0);
+    q[3 * j + 2] = A + B;
+  }
+}
+
+// ------------------------------------------------------------ collision of two cells, D3Q27 thermal
+// The update of collide_full with central moments (axis-by-axis transform of all of them), operation by operation
+// in the arithmetic of the one-cell kernel's FP32 form: same order, same products fused into an add,
+// so that its results are the same bits. Why here: a reacting flow turns rounding into differences
+// of another size (a fuel fraction of order 1/2 crossing zero, a face velocity changing sign: 1e-8 in u
+// becomes 1e-3 of the pressure fluctuation in 20 steps), so the arithmetic of reacting 3-D runs does not
+// change with the kernel that carries it.
+// ptxas fuses a packed product into the packed add that uses it, whatever the rounding modifiers and
+// -fmad say; mul_rn keeps a product's own rounding where it feeds an add: a fused multiply-add with a
+// -0 that ptxas cannot see through (constant memory).
+static __constant__ unsigned long long k_minus_zero2 = 0x8000000080000000ull;
+__device__ __forceinline__ F2 mul_rn(F2 a, F2 b) {
+  F2 z;
+  z.v = k_minus_zero2;
+  return fma_(a, b, z);
+}
+
+// One line of central moments about u (nu = -u, n2u = -2 u, uu = u u), forwards.
+__device__ __forceinline__ void line_fwd(F2& a, F2& b, F2& c, const F2 nu, const F2 n2u, const F2 uu) {
+  const F2 m0 = (a + b) + c, d = c - a, s = c + a;
+  a = m0;
+  b = fma_(nu, m0, d);
+  c = fma_(uu, m0, fma_(n2u, d, s));
+}
+// Back (u2 = 2 u), with the outer two values left at twice their size (exact; the final scale makes up
+// for it). RN: where the one-cell form rounds 2 u m1 by itself.
+template <bool RN>
+__device__ __forceinline__ void line_bwd(F2& a, F2& b, F2& c, const F2 u, const F2 u2, const F2 uu) {
+  const F2 m0 = a, m1 = b, m2 = c;
+  const F2 k1 = fma_(u, m0, m1);
+  const F2 k2 = fma_(uu, m0, RN ? m2 + mul_rn(u2, m1) : fma_(u2, m1, m2));
+  a = k2 - k1;
+  b = m0 - k2;
+  c = k2 + k1;
+}
+
+// Moments of order (A, B, C) of h_eq - w about u, to be subtracted: the seven terms of delta_eq.
+// e1, e2: -u_a and u_a u_a per axis.
+template <int J>
+__device__ __forceinline__ F2 delta_sum(const F2* e1, const F2* e2) {
+  constexpr int A = J % 3, B = J / 3 % 3, C = J / 9;
+  const F2 k3 = splat<F2>((double)(1.0f / 3.0f));
+  const F2 ex = A == 2 ? e2[0] : e1[0], ey = B == 2 ? e2[1] : e1[1], ez = C == 2 ? e2[2] : e1[2];
+  if constexpr (J == 8) return (mul_rn(ex, k3) + mul_rn(ey, k3)) + mul_rn(ex, ey);
+  F2 acc = splat<F2>(0.0);
+  bool any = false;
+  auto add = [&](F2 p, F2 r) {
+    acc = any ? fma_(p, r, acc) : p * r;
+    any = true;
+  };
+  if constexpr (A > 0 && B != 1 && C != 1) {
+    if constexpr (B == 2 && C == 2) add(ex * k3, k3);
+    else add(ex, k3);  // one of B, C is 2 in every order that comes here
+  }
+  if constexpr (B > 0 && A != 1 && C != 1) {
+    if constexpr (A == 2 && C == 2) add(ey * k3, k3);
+    else add(ey, k3);
+  }
+  if constexpr (C > 0 && A != 1 && B != 1) {
+    if constexpr (A == 2 && B == 2) add(ez, splat<F2>((double)((1.0f / 3.0f) * (1.0f / 3.0f))));
+    else add(ez, k3);
+  }
+  if constexpr (A > 0 && B > 0 && C != 1) {
+    if constexpr (C == 2) add(ex * ey, k3);
+    else add(ex, ey);
+  }
+  if constexpr (A > 0 && C > 0 && B != 1) {
+    if constexpr (B == 2) add(ex * k3, ez);
+    else add(ex, ez);
+  }
+  if constexpr (B > 0 && C > 0 && A != 1) {
+    if constexpr (A == 2) add(ey * k3, ez);
+    else add(ey, ez);
+  }
+  if constexpr (A > 0 && B > 0 && C > 0) add(ex * ey, ez);
+  return acc;
+}
+
+__device__ __forceinline__ void collide_central(F2* q, LBCell<3, F2, true>& c, const F2 nu3, const LBArgs<float>& a) {
+  typedef F2 V;
+  const V one = splat<V>(1.0), two = splat<V>(2.0), half = splat<V>(0.5), zero = splat<V>(0.0);
+  const V third = splat<V>((double)(1.0f / 3.0f)), ninth = splat<V>((double)(1.0f / 9.0f));
+  // weights by number of nonzero components of c_i
+  constexpr float W4[4] = {(float)wgt<3>(13), (float)wgt<3>(12), (float)wgt<3>(9), (float)wgt<3>(0)};
+  // their reciprocals times 1 / 2 per nonzero component (see line_bwd)
+  constexpr float F4[4] = {(float)(1.0 / wgt<3>(13)), 0.5f * (float)(1.0 / wgt<3>(12)),
+                           0.25f * (float)(1.0 / wgt<3>(9)), 0.125f * (float)(1.0 / wgt<3>(0))};
+  // ---- moments (Eq. 7)
+  V psum = zero, mx = zero, my = zero, mz = zero;
+#pragma unroll
+  for (int i = 0; i < 27; ++i) {
+    const double w = (double)(float)wgt<3>(i);
+    psum = fma_(splat<V>(w), q[i], psum);
+    if (cx(i)) mx = fma_(splat<V>(cx(i) * w), q[i], mx);
+    if (cy(i)) my = fma_(splat<V>(cy(i) * w), q[i], my);
+    if (cz(i)) mz = fma_(splat<V>(cz(i) * w), q[i], mz);
+  }
+  const V rho = c.rho, gx = c.gx, gy = c.gy, gz = c.gz, three = splat<V>(3.0);
+  const V inv_rho = rcp_(rho);
+  const V ux = mul_rn(three * mx, inv_rho), uy = mul_rn(three * my, inv_rho), uz = mul_rn(three * mz, inv_rho);
+  const V uxx = mul_rn(ux, ux), uyy = mul_rn(uy, uy), uzz = mul_rn(uz, uz);
+  const V usq = (uxx + uyy) + uzz;
+  const V udg = fma_(uz, gz, fma_(uy, gy, ux * gx));
+  const V rl3 = mul_rn(rho * c.lam, third);  // rho cs2 Lambda
+  const V k0 = fma_(third, udg, rl3);
+  const V S = fma_(half, k0, psum);
+  c.u[0] = ux;
+  c.u[1] = uy;
+  c.u[2] = uz;
+  c.usq = usq;
+  c.psum = psum;
+  c.rl3 = rl3;
+  const V tau0 = fma_(nu3, inv_rho, half);
+  // ---- central moments of w d about u
+  const V nux = zero - ux, nuy = zero - uy, nuz = zero - uz;
+  {
+    const V t3 = three * inv_rho, n2ux = two * nux;
+    V tw[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) tw[k] = t3 * splat<V>(W4[k]);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      const int k = (j % 3 != 1) + (j / 3 != 1);
+      const V xa = q[3 * j] - S, xb = q[3 * j + 1] - S, xc = q[3 * j + 2] - S;
+      const V A = tw[k + 1] * xa;
+      const V m0 = fma_(tw[k + 1], xc, fma_(tw[k], xb, A));
+      const V d = fma_(tw[k + 1], xc, zero - A), s = fma_(tw[k + 1], xc, A);
+      q[3 * j] = m0;
+      q[3 * j + 1] = fma_(nux, m0, d);
+      q[3 * j + 2] = fma_(uxx, m0, fma_(n2ux, d, s));
+    }
+    const V n2uy = two * nuy, n2uz = two * nuz;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int x = 0; x < 3; ++x) line_fwd(q[x + 9 * k], q[x + 3 + 9 * k], q[x + 6 + 9 * k], nuy, n2uy, uyy);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) line_fwd(q[j], q[j + 9], q[j + 18], nuz, n2uz, uzz);
+  }
+  // ---- half source (pre-conditioning) in moments of order 0..2
+  const V uxy = mul_rn(ux, uy), uxz = mul_rn(ux, uz), uyz = mul_rn(uy, uz);
+  {
+    const V h = splat<V>(1.5) * inv_rho;
+    const V u3[3] = {ux, uy, uz}, n3[3] = {nux, nuy, nuz}, g3[3] = {gx, gy, gz}, uu[3] = {uxx, uyy, uzz};
+    q[0] = fma_(h, k0, q[0]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int ja = i == 0 ? 1 : (i == 1 ? 3 : 9);
+      q[ja] = fma_(h, n3[i] * k0, q[ja]);
+      const V X = uu[i] + third, Z = fma_(two * g3[i], u3[i], udg);
+      q[2 * ja] = fma_(h, fma_(rl3, X, ninth * Z), q[2 * ja]);
+#pragma unroll
+      for (int b = i + 1; b < 3; ++b) {
+        const int jb = b == 1 ? 3 : 9;
+        const V Y = fma_(g3[i], u3[b], g3[b] * u3[i]);
+        q[ja + jb] = fma_(h, fma_(rl3 * u3[i], u3[b], ninth * Y), q[ja + jb]);
+      }
+    }
+  }
+  // deviation from the equilibrium, order 2
+  q[2] = q[2] + uxx;
+  q[6] = q[6] + uyy;
+  q[18] = q[18] + uzz;
+  q[4] = q[4] + uxy;
+  q[10] = q[10] + uxz;
+  q[12] = q[12] + uyz;
+  const V sum = (q[2] + q[6]) + q[18];
+  const V tr = mul_rn(third, sum);
+  // ---- relaxation time (Eq. 12, Smagorinsky)
+  V tau = tau0;
+  if (a.smag_k > 0.0f) {
+    const V nt = zero - third;
+    const V e0 = fma_(nt, sum, q[2]), e1 = fma_(nt, sum, q[6]), e2 = fma_(nt, sum, q[18]);
+    const V o2 = fma_(q[12], q[12], fma_(q[4], q[4], q[10] * q[10]));
+    const V n2 = fma_(two, o2, fma_(e2, e2, fma_(e0, e0, e1 * e1)));
+    tau = half * (tau0 + sqrt_pos(fma_(tau0, tau0, splat<V>(a.smag_k) * sqrt_rn(n2))));
+  }
+  const V o1 = one - rcp_(tau), obt = splat<V>(1.0f - a.omega_b) * tr;
+  // ---- relaxed second-order moments and the higher ones without cumulants
+  const V sxx = fma_(o1, q[2] - tr, obt), syy = fma_(o1, q[6] - tr, obt), szz = fma_(o1, q[18] - tr, obt);
+  const V sxy = mul_rn(o1, q[4]), sxz = mul_rn(o1, q[10]), syz = mul_rn(o1, q[12]);
+  const V tx = third + sxx, ty = third + syy, tz = third + szz;
+  const V s2xy = two * sxy, s2xz = two * sxz, sxxyy = mul_rn(sxx, syy);
+  const V e1[3] = {nux, nuy, nuz}, e2[3] = {uxx, uyy, uzz};
+  V Dd = fma_(ninth, (sxx + syy) + szz, third * fma_(szz, sxx, fma_(syy, szz, sxxyy)));
+  Dd = fma_(sxxyy, szz, Dd);
+  Dd = fma_(two, fma_(tz * sxy, sxy, fma_(tx * syz, syz, (ty * sxz) * sxz)), Dd);
+  Dd = fma_((splat<V>(8.0) * sxy) * sxz, syz, Dd);
+  q[26] = Dd - delta_sum<26>(e1, e2);
+  q[2] = sxx - uxx;
+  q[6] = syy - uyy;
+  q[18] = szz - uzz;
+  q[4] = sxy - uxy;
+  q[10] = sxz - uxz;
+  q[12] = syz - uyz;
+  q[5] = zero - delta_sum<5>(e1, e2);
+  q[7] = zero - delta_sum<7>(e1, e2);
+  q[11] = zero - delta_sum<11>(e1, e2);
+  q[13] = zero - delta_sum<13>(e1, e2);
+  q[15] = zero - delta_sum<15>(e1, e2);
+  q[19] = zero - delta_sum<19>(e1, e2);
+  q[21] = zero - delta_sum<21>(e1, e2);
+  q[14] = fma_(s2xy, sxz, tx * syz) - delta_sum<14>(e1, e2);
+  q[16] = fma_(s2xy, syz, ty * sxz) - delta_sum<16>(e1, e2);
+  q[22] = fma_(s2xz, syz, tz * sxy) - delta_sum<22>(e1, e2);
+  q[8] = fma_(s2xy, sxy, mul_rn(third, sxx + syy) + sxxyy) - delta_sum<8>(e1, e2);
+  q[20] = fma_(s2xz, sxz, fma_(sxx, szz, third * (sxx + szz))) - delta_sum<20>(e1, e2);
+  q[24] = fma_(two * syz, syz, fma_(syy, szz, third * (syy + szz))) - delta_sum<24>(e1, e2);
+  q[17] = zero - delta_sum<17>(e1, e2);
+  q[23] = zero - delta_sum<23>(e1, e2);
+  q[25] = zero - delta_sum<25>(e1, e2);
+  // ---- back to populations
+  {
+    const V u2x = two * ux, u2y = two * uy, u2z = two * uz;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) line_bwd<false>(q[j], q[j + 9], q[j + 18], uz, u2z, uzz);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        if (k == 1) line_bwd<false>(q[x + 9 * k], q[x + 3 + 9 * k], q[x + 6 + 9 * k], uy, u2y, uyy);
+        else line_bwd<true>(q[x + 9 * k], q[x + 3 + 9 * k], q[x + 6 + 9 * k], uy, u2y, uyy);
+      }
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      if (j % 3 == 1) line_bwd<false>(q[3 * j], q[3 * j + 1], q[3 * j + 2], ux, u2x, uxx);
+      else line_bwd<true>(q[3 * j], q[3 * j + 1], q[3 * j + 2], ux, u2x, uxx);
+    }
+  }
+  // ---- post-collision (Eq. 8): scale, S and the half source
+  V fac[4];
+  {
+    const V rho3 = rho * third;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) fac[k] = rho3 * splat<V>(F4[k]);
+  }
+  const V hu = splat<V>(-0.5) * usq, ngx = zero - gx, ngy = zero - gy, ngz = zero - gz;
+  auto out = [&](int i, int k, V t, V cu, V cg) {
+    const V e = k ? fma_(t, cu, cu) + hu : hu;
+    const V E = fma_(e, cg - udg, rl3);
+    q[i] = fma_(half, E, fma_(fac[k], q[i], S));
+  };
+  out(13, 0, zero, zero, zero);
+#pragma unroll
+  for (int i = 0; i < 13; ++i) {
+    // direction i and its opposite, which share the product 1.5 c.u
+    const int k = (cx(i) != 0) + (cy(i) != 0) + (cz(i) != 0);
+    V cu = zero, cg = zero, nu_ = zero, ng = zero;
+    bool any = false;
+    auto add = [&](int s, V u, V nu, V g, V n) {
+      const V pu = s > 0 ? u : nu, mu = s > 0 ? nu : u, pg = s > 0 ? g : n, mg = s > 0 ? n : g;
+      cu = any ? cu + pu : pu;
+      nu_ = any ? nu_ + mu : mu;
+      cg = any ? cg + pg : pg;
+      ng = any ? ng + mg : mg;
+      any = true;
+    };
+    if (cx(i)) add(cx(i), ux, nux, gx, ngx);
+    if (cy(i)) add(cy(i), uy, nuy, gy, ngy);
+    if (cz(i)) add(cz(i), uz, nuz, gz, ngz);
+    const V t = splat<V>(1.5) * cu;
+    out(i, k, t, cu, cg);
+    const V e = fma_(t, cu, nu_) + hu;
+    q[26 - i] = fma_(half, fma_(e, ng - udg, rl3), fma_(fac[k], q[26 - i], S));
+  }
+}
+
+
+// ------------------------------------------------------------------ pull streaming of one cell
+// raw[i] = stored q_i = g_i / w_i - P_ref from r - c_i, or the opposite population of the cell itself
+// on bounce-back links; rho_p, rho_m: density at r + e_a, r - e_a (the cell's own where the link there
+// is not a plain pull). Offsets fit in 32 bits (checked at init). Per-axis offsets to the minus /
+// plus neighbour wrap on periodic faces (a plain pull across a non-periodic face never happens: those
+// links are bounce-back, inlet or outlet links). All loads are issued before any is converted.
+template <int D, typename S, typename R, bool THERMAL>
+__device__ __forceinline__ void pull_cell(const LBArgs<R>& a, int r, int x, int y, int z, uint32_t lw, S* raw,
+                                          R* rho_p, R* rho_m) {
+  constexpr int Q = Lat<D>::Q;
+  const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz, Ni = a.geo.N;
+  const S* __restrict__ gin = (const S*)a.g_in;
+  const int sy_ = nx, sz_ = nx * ny;
+  const int oxm = x > 0 ? -1 : nx - 1, oxp = x < nx - 1 ? 1 : 1 - nx;
+  const int oym = y > 0 ? -sy_ : (ny - 1) * sy_, oyp = y < ny - 1 ? sy_ : (1 - ny) * sy_;
+  const int ozm = z > 0 ? -sz_ : (nz - 1) * sz_, ozp = z < nz - 1 ? sz_ : (1 - nz) * sz_;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int ci = cx(i), cj = cy(i), ck = (D == 3) ? cz(i) : 0;
+    // source r - c_i
+    const int s = r + (ci == 1 ? oxm : (ci == -1 ? oxp : 0)) + (cj == 1 ? oym : (cj == -1 ? oyp : 0)) +
+                  (ck == 1 ? ozm : (ck == -1 ? ozp : 0));
+    const bool link = (lw >> i) & 1u;
+    raw[i] = ld_raw<S>(gin + (link ? (Q - 1 - i) * Ni + r : i * Ni + s));
+    if constexpr (THERMAL) {
+      if (ci * ci + cj * cj + ck * ck == 1 && !link) {
+        // direction -e_a pulls from r + e_a; +e_a pulls from r - e_a
+        const R rs = ldg(a.rho + s);
+        if (ci == -1) rho_p[0] = rs;
+        if (ci == 1) rho_m[0] = rs;
+        if (cj == -1) rho_p[1] = rs;
+        if (cj == 1) rho_m[1] = rs;
+        if (D == 3 && ck == -1) rho_p[2] = rs;
+        if (D == 3 && ck == 1) rho_m[2] = rs;
+      }
+    }
+  }
+}
+
+// Inlet and outlet rules of one cell on its pulled populations q.
+template <int D, typename R>
+__device__ __forceinline__ void face_rules(const LBArgs<R>& a, int r, int x, int y, int z, uint32_t lw, R rho, R* q) {
+  constexpr int Q = Lat<D>::Q;
+  const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz;
+  // moving-wall term of the low-x inlet: g_i += 2 w_i rho (c_i . u_w)
+  if (x == 0 && a.geo.bc_lo[0] == BC_INLET) {
+    const int f = y + ny * z;
+    const int nf = ny * nz;
+    const R uw0 = ldg(a.inlet_u + f), uw1 = ldg(a.inlet_u + nf + f);
+    const R uw2 = (D == 3) ? ldg(a.inlet_u + 2 * nf + f) : R(0);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      if (cx(i) == 1) {
+        if ((lw >> i) & 1u) {
+          const R cu = uw0 + (R)cy(i) * uw1 + ((D == 3) ? (R)cz(i) * uw2 : R(0));
+          q[i] += R(2) * rho * cu;
+        }
+      }
+    }
+  }
+  // pressure outlet (anti-bounce-back at the half-way face, P_h = P_ref):
+  // g_i = -g*_opp + 2 w_i (P_ref + rho (1.5 (c_i.u)^2 - 0.5 u^2)), u of the previous step
+  if (x == nx - 1 && a.geo.bc_hi[0] == BC_OUTLET) {
+    const size_t N = (size_t)a.geo.N;
+    const R vx = a.u_in[r], vy = a.u_in[N + r], vz = (D == 3) ? a.u_in[2 * N + r] : R(0);
+    const R vv = vx * vx + vy * vy + vz * vz;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      if (cx(i) == -1) {
+        if ((lw >> i) & 1u) {
+          const R cu = -vx + (R)cy(i) * vy + ((D == 3) ? (R)cz(i) * vz : R(0));
+          q[i] = -q[i] + rho * (R(3) * cu * cu - vv);
+        }
+      }
+    }
+  }
+}
+
 // WALLS = false: every fluid cell except those flagged LINK_WALL, one block row per (y, z).
 // WALLS = true: the flagged cells only, one thread per entry of the wall list, with the
 // interpolated bounce-back fix-up compiled in (so that it costs the other cells no registers).
@@ -191,8 +790,8 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
     y = (r / nx) % ny;
     z = r / (nx * ny);
   } else {
-    // one block row of LB_BLOCK cells along x; y and z come from the grid (no integer division)
-    x = blockIdx.x * LB_BLOCK + threadIdx.x;
+    // one block row of cells along x; y and z come from the grid (no integer division)
+    x = blockIdx.x * blockDim.x + threadIdx.x;
     y = blockIdx.y;
     z = blockIdx.z;
     if (x >= nx) return;
@@ -340,6 +939,29 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
         }
       }
     }
+  }
+
+  if constexpr (COLL == COLL_CUMULANT_FULL && sizeof(R) == 8) {
+    LBCell<D, R, THERMAL> c;
+    c.rho = rho;
+    c.lam = lam;
+    if constexpr (THERMAL) {
+      c.gx = R(0.5) * (rho_p[0] - rho_m[0]);
+      c.gy = R(0.5) * (rho_p[1] - rho_m[1]);
+      c.gz = (D == 3) ? R(0.5) * (rho_p[2] - rho_m[2]) : R(0);
+    }
+    collide_full<D, R, THERMAL, R>(q, c, R(3) * a.nu_lat * (THERMAL ? pw<R>(T_early * a.T_ref_inv, a.mu_exp) : R(1)), a);
+    S* __restrict__ gout = (S*)a.g_out;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) st_pop<S, R>(gout + i * Ni + r, q[i]);
+    if (a.write_u || outlet_cell) {
+      a.u[r] = c.u[0];
+      a.u[N + r] = c.u[1];
+      if (D == 3) a.u[2 * N + r] = c.u[2];
+    }
+    if (a.ph_out) a.ph_out[r] = a.P_ref + c.psum + R(0.5) * c.rl3;
+    if (!isfinite(c.usq)) atomicOr(a.flag, 1);
+    return;
   }
 
   // ---------------------------------------------------------------- moments (Eq. 7)
@@ -536,14 +1158,243 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
   if (!isfinite(usq)) atomicOr(a.flag, 1);
 }
 
+
+// ------------------------------------------------------------------ two cells per thread
+// Stream-collide of FP32 arithmetic with full relaxation of the orders 3..6 (the default rates): a
+// thread owns the cells r, r + 1 (r even) of the linear index and runs them through packed
+// instructions (packed.cuh). The one-cell kernel waited on instruction issue (70% of the slots, 44%
+// of DRAM peak); here each arithmetic instruction serves two cells, the populations of c_x = 0 and
+// all stores move 64 bits (VEC), and address arithmetic is shared: 86.5 M -> 44.9 M warp
+// instructions on the reactive 192x96x96 case (30.3 M with collide_full). Rows of any length fill every warp, since the threads follow the linear
+// index (with one block row per grid row, 135 cells took 256 threads).
+// Before -> after per launch, FP32 / FP16 populations: cold swirl 256x128x128 180 -> 138 / 175 -> 104 us
+// and periodic box 161x129x97 112 -> 72 us (90% of the copy peak by its 217 B per cell; bound by DRAM
+// and its latency: 35% issue); reactive swirl 384x192x192 (collide_central) 655 -> 577 / 672 -> 554 us,
+// bound by the FP32 pipe (57% busy) and load latency at 14 warps per SM. L2 prefetch hints of 64 to 256
+// bytes, none, and streaming stores on FP32 differ by less than 2%; loads that do not allocate in L1
+// cost 14-25% (the x-shifted pulls of a pair share lines there).
+// VEC: nx even and every array aligned to two elements, else each element is loaded and stored by
+// itself. Cells with boundary links or on periodic faces pull one by one (pull_cell) in the warps
+// that hold such cells; the others take the plain offsets. (Taking plain loads there for each
+// direction without links in the warp, behind 27 uniform branches, was level in FP32 and 10% slower
+// in FP16: the branches keep the loads of a cell from being in flight together. Prefetching the
+// populations of a later block into L2 was 2-30% slower.)
+constexpr int LP_BLOCK = 64;
+// resident blocks the registers are sized for: 128 registers thermal (102 registers spill, 13% slower),
+// 96 isothermal (cold swirl 256x128x128 FP16 111 -> 104 us per step against 128 registers). Blocks of 64
+// against 128 threads are 1% faster.
+constexpr int LP_MIN_THERMAL = 8, LP_MIN_ISOTHERMAL = 10;
+
+template <typename S> __device__ __forceinline__ void ld_raw2(const S* p, S& a, S& b);
+template <> __device__ __forceinline__ void ld_raw2<float>(const float* p, float& a, float& b) {
+  asm("ld.global.nc.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "l"(p));
+}
+template <> __device__ __forceinline__ void ld_raw2<__half>(const __half* p, __half& a, __half& b) {
+  unsigned short u, v;
+  asm("ld.global.nc.L2::256B.v2.u16 {%0, %1}, [%2];" : "=h"(u), "=h"(v) : "l"(p));
+  a = __ushort_as_half(u);
+  b = __ushort_as_half(v);
+}
+__device__ __forceinline__ void st2(float* p, F2 v) { *reinterpret_cast<float2*>(p) = make_float2(lo(v), hi(v)); }
+__device__ __forceinline__ void st_pop2(float* p, F2 v) { st2(p, v); }
+__device__ __forceinline__ void st_pop2(__half* p, F2 v) {
+  const __half2 h = __floats2half2_rn(lo(v), hi(v));
+  __stcs(reinterpret_cast<unsigned int*>(p), *reinterpret_cast<const unsigned int*>(&h));
+}
+template <bool VEC> __device__ __forceinline__ F2 ld_pair(const float* p, bool two) {
+  if constexpr (VEC) {
+    const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+    return pack2(v.x, v.y);
+  }
+  return pack2(__ldg(p), __ldg(p + (two ? 1 : 0)));
+}
+
+template <int D, typename S, bool THERMAL, bool VEC>
+__global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_ISOTHERMAL) lb_pair_kernel(const LBArgs<float> a) {
+  constexpr int Q = Lat<D>::Q;
+  constexpr uint32_t LINKS = (1u << Q) - 1u;
+  const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz, N = a.geo.N;
+  const int r = 2 * (blockIdx.x * LP_BLOCK + threadIdx.x);
+  if (r >= N) return;
+  const bool two = VEC || r + 1 < N;  // the last cell of an odd grid has no partner
+  F2 rho = splat<F2>(1.0), lam = splat<F2>(0.0), T = splat<F2>(1.0);
+  if constexpr (THERMAL) {
+    rho = ld_pair<VEC>(a.rho + r, two);
+    lam = ld_pair<VEC>(a.lam + r, two);
+    T = ld_pair<VEC>(a.T + r, two);
+  }
+  const uint32_t lw0 = __ldg(a.links + r), lw1 = two ? __ldg(a.links + r + 1) : 0u;
+  // cells this launch updates: fluid ones, except those of the interpolated-wall list
+  const bool act0 = (lw0 >> 30) == 2u, act1 = (lw1 >> 30) == 2u;
+  if (!act0 && !act1) return;
+  const int row = a.div_nx.div(r), z0 = D == 3 ? a.div_ny.div(row) : 0;
+  const int x0 = r - row * nx, y0 = D == 3 ? row - z0 * ny : row;
+  const bool plain = act0 && act1 && ((lw0 | lw1) & LINKS) == 0u && x0 > 0 && x0 + 2 < nx && y0 > 0 && y0 < ny - 1 &&
+                     (D == 2 || (z0 > 0 && z0 < nz - 1));
+  S raw0[Q], raw1[Q];
+  F2 gx = splat<F2>(0.0), gy = gx, gz = gx;
+  F2 q[Q];
+  bool out0 = false, out1 = false;  // outlet cells
+  if (__all_sync(__activemask(), plain)) {
+    const S* __restrict__ gin = (const S*)a.g_in;
+    const int sy_ = nx, sz_ = nx * ny;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const int ci = cx(i), cj = cy(i), ck = (D == 3) ? cz(i) : 0;
+      const S* p = gin + (size_t)i * N + (unsigned)(r - cj * sy_ - ck * sz_) - ci;
+      if (VEC && ci == 0) {
+        ld_raw2<S>(p, raw0[i], raw1[i]);
+      } else {
+        raw0[i] = ld_raw<S>(p);
+        raw1[i] = ld_raw<S>(p + 1);
+      }
+    }
+    if constexpr (THERMAL) {
+      const float left = ldg(a.rho + r - 1), right = ldg(a.rho + r + 2);
+      const F2 yp = ld_pair<VEC>(a.rho + r + sy_, true), ym = ld_pair<VEC>(a.rho + r - sy_, true);
+      gx = splat<F2>(0.5) * (pack2(hi(rho), right) - pack2(left, lo(rho)));
+      gy = splat<F2>(0.5) * (yp - ym);
+      if constexpr (D == 3) {
+        const F2 zp = ld_pair<VEC>(a.rho + r + sz_, true), zm = ld_pair<VEC>(a.rho + r - sz_, true);
+        gz = splat<F2>(0.5) * (zp - zm);
+      }
+    }
+    pdl_wait();
+#pragma unroll
+    for (int i = 0; i < Q; ++i) q[i] = pack2(cvt_pop<S, float>(raw0[i]), cvt_pop<S, float>(raw1[i]));
+  } else {
+    // cells on walls, inlets, outlets, next to solids or on periodic faces are in this warp
+    const bool wrap = x0 + 1 == nx;
+    const int x1 = wrap ? 0 : x0 + 1, y1 = wrap ? (y0 + 1 == ny && D == 3 ? 0 : y0 + 1) : y0;
+    const int z1 = (D == 3 && wrap && y0 + 1 == ny) ? z0 + 1 : z0, r1 = two ? r + 1 : r;
+    float rp[3], rm[3], sp[3], sm[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      rp[d] = rm[d] = lo(rho);
+      sp[d] = sm[d] = hi(rho);
+    }
+    // a cell that is not updated reads its own populations
+    pull_cell<D, S, float, THERMAL>(a, r, x0, y0, z0, act0 ? lw0 : LINKS, raw0, rp, rm);
+    pull_cell<D, S, float, THERMAL>(a, r1, x1, y1, z1, act1 ? lw1 : LINKS, raw1, sp, sm);
+    if constexpr (THERMAL) {
+      gx = splat<F2>(0.5) * (pack2(rp[0], sp[0]) - pack2(rm[0], sm[0]));
+      gy = splat<F2>(0.5) * (pack2(rp[1], sp[1]) - pack2(rm[1], sm[1]));
+      if constexpr (D == 3) gz = splat<F2>(0.5) * (pack2(rp[2], sp[2]) - pack2(rm[2], sm[2]));
+    }
+    pdl_wait();
+    float p0[Q], p1[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      p0[i] = cvt_pop<S, float>(raw0[i]);
+      p1[i] = cvt_pop<S, float>(raw1[i]);
+    }
+    if (act0) face_rules<D, float>(a, r, x0, y0, z0, lw0, lo(rho), p0);
+    if (act1) face_rules<D, float>(a, r1, x1, y1, z1, lw1, hi(rho), p1);
+    out0 = x0 == nx - 1 && a.geo.bc_hi[0] == BC_OUTLET;
+    out1 = x1 == nx - 1 && a.geo.bc_hi[0] == BC_OUTLET;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) q[i] = pack2(p0[i], p1[i]);
+  }
+  LBCell<D, F2, THERMAL> c;
+  c.rho = rho;
+  c.lam = lam;
+  F2 nu3 = splat<F2>(3.0f * a.nu_lat);
+  if constexpr (THERMAL) {
+    c.lam = lam + splat<F2>(a.pth->lb_lam);
+    c.gx = gx;
+    c.gy = gy;
+    c.gz = gz;
+    const F2 t = T * splat<F2>(a.T_ref_inv);
+    nu3 = nu3 * pack2(pw<float>(lo(t), a.mu_exp), pw<float>(hi(t), a.mu_exp));
+  }
+  if constexpr (D == 3 && THERMAL) collide_central(q, c, nu3, a);
+  else collide_full<D, F2, THERMAL, float>(q, c, nu3, a);
+
+  S* __restrict__ gout = (S*)a.g_out;
+  const bool both = act0 && act1;
+  if (VEC && both) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) st_pop2(gout + (size_t)i * N + (unsigned)r, q[i]);
+    if (a.write_u) {
+#pragma unroll
+      for (int d = 0; d < D; ++d) st2(a.u + (size_t)d * N + (unsigned)r, c.u[d]);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      S* p = gout + (size_t)i * N + (unsigned)r;
+      if (act0) st_pop<S, float>(p, lo(q[i]));
+      if (act1) st_pop<S, float>(p + 1, hi(q[i]));
+    }
+    if (a.write_u) {
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        float* p = a.u + (size_t)d * N + (unsigned)r;
+        if (act0) p[0] = lo(c.u[d]);
+        if (act1) p[1] = hi(c.u[d]);
+      }
+    }
+  }
+  if (!a.write_u) {  // the outlet rule of the next step reads u
+    if (out0 && act0)
+      for (int d = 0; d < D; ++d) a.u[(size_t)d * N + r] = lo(c.u[d]);
+    if (out1 && act1)
+      for (int d = 0; d < D; ++d) a.u[(size_t)d * N + r + 1] = hi(c.u[d]);
+  }
+  if (a.ph_out) {
+    const F2 p = fma_(splat<F2>(0.5), c.rl3, splat<F2>(a.P_ref) + c.psum);
+    if (act0) a.ph_out[r] = lo(p);
+    if (act1) a.ph_out[r + 1] = hi(p);
+  }
+  if ((act0 && !isfinite(lo(c.usq))) || (act1 && !isfinite(hi(c.usq)))) atomicOr(a.flag, 1);
+}
+
+// Whether every array of a pair launch may be accessed two elements at a time.
+template <typename S> bool pair_aligned(const LBArgs<float>& a, bool thermal) {
+  uintptr_t f = (uintptr_t)a.u | (uintptr_t)a.ph_out;
+  if (thermal) f |= (uintptr_t)a.rho | (uintptr_t)a.lam | (uintptr_t)a.T;
+  return a.geo.nx % 2 == 0 && f % 8 == 0 && ((uintptr_t)a.g_in | (uintptr_t)a.g_out) % (2 * sizeof(S)) == 0;
+}
+
+template <int D, typename S, bool THERMAL>
+cudaError_t launch_pair(LBArgs<float> a, cudaStream_t st, bool pdl) {
+  a.div_nx = FastDiv((uint32_t)a.geo.nx);
+  a.div_ny = FastDiv((uint32_t)a.geo.ny);
+  const int pairs = (a.geo.N + 1) / 2;
+  const dim3 grid((pairs + LP_BLOCK - 1) / LP_BLOCK);
+  if (pair_aligned<S>(a, THERMAL))
+    return launch_ex<LBArgs<float>>(lb_pair_kernel<D, S, THERMAL, true>, grid, dim3(LP_BLOCK), st, pdl, a);
+  return launch_ex<LBArgs<float>>(lb_pair_kernel<D, S, THERMAL, false>, grid, dim3(LP_BLOCK), st, pdl, a);
+}
+
+// The stream-collide of every cell not on the wall list. FP32 arithmetic at the default rates: two cells
+// per thread in 3-D, and in 2-D from PAIR_MIN_2D cells on; below that the grid does not fill the GPU
+// with pairs and the longer threads cost what the fewer instructions save (chamber step, one cell / two:
+// 256x64 13.47 / 13.53 us, 512x128 14.48 / 14.48, 600x200 17.58 / 16.59, 1024x256 27.20 / 25.07; 3-D
+// gains at every size, e.g. periodic box of 82,615 cells 10.35 / 5.47 us). Otherwise one cell per thread.
+constexpr int PAIR_MIN_2D = 100000;
+template <int D, typename S, typename R, bool THERMAL, int COLL>
+cudaError_t launch_cells(const LBArgs<R>& a, cudaStream_t st, bool pdl) {
+  constexpr bool PAIR = COLL == COLL_CUMULANT_FULL && sizeof(R) == 4;
+  if constexpr (PAIR) {
+    if (D == 3 || a.geo.N >= PAIR_MIN_2D) return launch_pair<D, S, THERMAL>(a, st, pdl);
+  }
+  if constexpr (!PAIR || D == 2) {
+    // blocks of one warp where larger ones would leave SMs empty (planar flame 256x8 FP64, with the FD
+    // update spread the same way: 122 -> 34 us per step)
+    const int block = a.geo.N < 32768 ? 32 : LB_BLOCK;
+    const dim3 grid((a.geo.nx + block - 1) / block, a.geo.ny, a.geo.nz);
+    return launch_ex<LBArgs<R>>(lb_step_kernel<D, S, R, THERMAL, COLL, false>, grid, dim3(block), st, pdl, a);
+  }
+}
+
 // pdl: the kernel may start while the one before it in the stream (the thermodynamic-pressure
 // update) runs; it reads that kernel's state after pdl_wait.
 template <int D, typename S, typename R>
 cudaError_t launch_lb(const LBArgs<R>& a, int thermal, int coll, cudaStream_t st, bool pdl) {
-  const dim3 grid((a.geo.nx + LB_BLOCK - 1) / LB_BLOCK, a.geo.ny, a.geo.nz);
 #define LB_LAUNCH(TH, CO)                                                                         \
   do {                                                                                            \
-    cudaError_t e_ = launch_ex<LBArgs<R>>(lb_step_kernel<D, S, R, TH, CO, false>, grid, dim3(LB_BLOCK), st, pdl, a); \
+    cudaError_t e_ = launch_cells<D, S, R, TH, CO>(a, st, pdl);                                   \
     if (e_ != cudaSuccess) return e_;                                                             \
     if (a.n_wall > 0)                                                                             \
       lb_step_kernel<D, S, R, TH, CO, true><<<(a.n_wall + LB_BLOCK - 1) / LB_BLOCK, LB_BLOCK, 0, st>>>(a); \
