@@ -362,8 +362,15 @@ cudaError_t run_lb(lbm_ctx* c, int cur, bool want_out) {
 // the tiled update applies (3-D FP32, constant heat capacity, grid and chemistry it supports)
 bool use_tiled(const lbm_ctx* c) { return c->tiled && !c->fdc_f.varcp && !c->fdc_f.mixavg; }
 
+// the one-warp-per-field update applies (small 2-D FP64, none of the options)
+bool use_split(const lbm_ctx* c) {
+  return c->f64 && c->D == 2 && c->N <= (size_t)FD_SPLIT_MAX && !c->fdc_d.varcp && !c->fdc_d.mixavg &&
+         !c->n_fd_wall_rows;
+}
+
 // partial slots of the P_th reduction written by one FD update
 int fd_slots(const lbm_ctx* c) {
+  if (use_split(c)) return fd_split_blocks(c->geo);
   if (!use_tiled(c)) return c->nblocks_fd;
   return c->nblocks_tiled + (int)((c->n_fd_wall_rows + FD_BLOCK - 1) / FD_BLOCK);
 }
@@ -371,6 +378,7 @@ int fd_slots(const lbm_ctx* c) {
 cudaError_t run_fd(lbm_ctx* c, int cur, bool sensor_pass) {
   if (c->f64) {
     auto a = make_fd_args<double>(c, cur);
+    if (!sensor_pass && use_split(c)) return launch_fd_split(a, c->st);
     return c->D == 2 ? launch_fd<2, double>(a, c->st, sensor_pass) : launch_fd<3, double>(a, c->st, sensor_pass);
   }
   auto a = make_fd_args<float>(c, cur);
@@ -534,8 +542,9 @@ lbm_status lbm_init(const lbm_config* cfg, lbm_ctx** out) {
     ctx->tiled = fd_tiled_create();
     if (!ctx->tiled) ok = false;
   }
-  ok = ok && (ctx->partials = dalloc(ctx, (size_t)std::max(ctx->nblocks_fd * (ctx->tiled ? 2 : 1),
-                                                           ctx->nblocks_init) * 16));
+  const int n_split = c.thermal && use_split(ctx) ? fd_split_blocks(ctx->geo) : 0;
+  ok = ok && (ctx->partials = dalloc(ctx, (size_t)std::max({ctx->nblocks_fd * (ctx->tiled ? 2 : 1),
+                                                            ctx->nblocks_init, n_split}) * 16));
   ok = ok && (ctx->pth_stage = dalloc(ctx, (size_t)pth_stage_words() * 8));
   ok = ok && (ctx->pth_counter = (unsigned int*)dalloc(ctx, 16));
   if (c.thermal) {
@@ -1230,7 +1239,12 @@ lbm_status seg_recompute(lbm_ctx* ctx, const void* checkpoint, int n, R* ws, cud
       fdf.Y_out = last ? (R*)ctx->Y[other] : sk1 + 12 * N;
       fdf.rho_out = rho_of(k);
       fdf.lam_out = rho_of(k) + N;
-      CK((launch_fd<2, R>(fdf, st, false)), "segment recompute (FD)");
+      // the forward step's own update (the sweep reproduces its states bit for bit)
+      if constexpr (sizeof(R) == 8) {
+        CK((use_split(ctx) ? launch_fd_split(fdf, st) : launch_fd<2, R>(fdf, st, false)), "segment recompute (FD)");
+      } else {
+        CK((launch_fd<2, R>(fdf, st, false)), "segment recompute (FD)");
+      }
     }
     if (!last) {
       LBArgs<R> lbf = make_lb_args<R>(ctx, ctx->cur, false);

@@ -23,6 +23,11 @@ cudaError_t fd_tiled_setup(FDTiledMaps& m, const Geo& g, int K, void* const T[2]
 int fd_tiled_blocks(const FDTiledMaps& m);
 cudaError_t launch_fd_tiled(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st);
 
+// fd_split.cu: FD update of small 2-D FP64 grids, one warp per field (no options, no wall weights)
+constexpr int FD_SPLIT_MAX = 32768;
+int fd_split_blocks(const Geo& g);
+cudaError_t launch_fd_split(const FDArgs<double>& a, cudaStream_t st);
+
 // aux_kernels.cu
 cudaError_t launch_links(int D, const Geo& g, const uint8_t* mask, uint32_t* out, cudaStream_t st);
 cudaError_t launch_stencil_words(int D, const Geo& g, const uint8_t* mask, uint32_t* out, cudaStream_t st);
