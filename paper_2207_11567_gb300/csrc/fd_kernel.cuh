@@ -506,14 +506,9 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
 
 // NK, NR > 0: species and reaction counts known at compile time (loops unroll exactly);
 // NK = NR = 0: counts read from the constants at run time.
-#ifndef HLBM_FD_MIN_BLOCKS
-#define HLBM_FD_MIN_BLOCKS 4  // FP32: resident blocks per SM the register budget is sized for
-#endif
-#ifndef HLBM_FD_VCP_MIN_BLOCKS
-#define HLBM_FD_VCP_MIN_BLOCKS 4  // the same for the variable heat-capacity variant (measured: 2 blocks 2.24 ms, 3 blocks 1.72 ms, 4 blocks 1.60 ms per C4 launch)
-#endif
-template <int D, typename R, int NK, int NR, int VDEG = 0, bool MIX = false>
-__global__ void __launch_bounds__(FD_BLOCK, sizeof(R) == 4 ? (VDEG > 0 ? HLBM_FD_VCP_MIN_BLOCKS : HLBM_FD_MIN_BLOCKS) : 1)
+// MINB: FP32 resident blocks per SM that the register budget is sized for.
+template <int D, typename R, int NK, int NR, int VDEG = 0, bool MIX = false, int MINB = 4>
+__global__ void __launch_bounds__(FD_BLOCK, sizeof(R) == 4 ? MINB : 1)
     fd_step_kernel(const FDArgs<R> a) {
   const FDConst<R>& c = a.c;
   const Geo& g = a.geo;
