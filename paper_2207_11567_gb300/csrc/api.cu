@@ -54,6 +54,7 @@ struct lbm_ctx {
   int nblocks_fd = 0;    // partial slots written by fd_step_kernel over the whole grid
   FDTiledMaps* tiled = nullptr;  // tiled FD update (3-D FP32), nullptr where it does not apply
   int nblocks_tiled = 0;         // partial slots written by the tiled update
+  int* fd_tiles = nullptr;       // its tiles that hold fluid
   size_t n_fd_wall_rows = 0;     // cells with ghost-point wall weights (fd_step_kernel, walls only)
   int* fd_wall_list = nullptr;   // those cells, ascending (the tiled update's walls-only launch)
   size_t fd_wall_list_cap = 0;
@@ -567,8 +568,12 @@ lbm_status lbm_init(const lbm_config* cfg, lbm_ctx** out) {
     CK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, ctx->dev), "device attribute");
     CK(fd_tiled_setup(*ctx->tiled, ctx->geo, ctx->K, ctx->T, ctx->Y, ctx->Floc, ctx->u, ctx->sword, n_sm),
        "tensor maps of the tiled FD update");
-    ctx->nblocks_tiled = fd_tiled_blocks(*ctx->tiled);
-    if (ctx->nblocks_tiled > ctx->nblocks_fd) return fail(ctx, LBM_ERR_ARG, "tiled FD grid too large");
+    const int nt = fd_tiled_tiles(*ctx->tiled, ctx->geo);
+    if (nt > ctx->nblocks_fd) return fail(ctx, LBM_ERR_ARG, "tiled FD grid too large");
+    if (!(ctx->fd_tiles = (int*)dalloc(ctx, (size_t)nt * sizeof(int)))) {
+      dfree_all(ctx);
+      return fail(ctx, LBM_ERR_ALLOC, "device allocation failed");
+    }
   }
   for (int b = 0; b < 2; ++b)
     if (ctx->Floc[b]) CK(cudaMemsetAsync(ctx->Floc[b], 0, N * ctx->F, ctx->st), "memset");
@@ -746,6 +751,10 @@ lbm_status lbm_set_geometry(lbm_ctx* ctx, const uint8_t* mask, const double* inl
   size_t nfl = 0;
   for (size_t i = 0; i < N; ++i) nfl += hm[i] == 0;
   ctx->n_fluid = nfl;
+  if (ctx->tiled) {
+    CK(fd_tiled_set_mask(*ctx->tiled, ctx->geo, hm.data(), ctx->fd_tiles, ctx->st), "tile list");
+    ctx->nblocks_tiled = fd_tiled_blocks(*ctx->tiled);
+  }
   ctx->have_geo = true;
   ctx->floc_ok = false;
   ctx->n_wall = 0;  // the rebuilt link words carry no interpolated walls

@@ -159,21 +159,14 @@ cudaError_t launch_ex(void (*kern)(Arg), dim3 grid, dim3 block, cudaStream_t st,
 template <typename R> __device__ __forceinline__ R ldg(const R* p) { return __ldg(p); }
 
 // ---------------------------------------------------------------------------- fixed point
-// x * 2^32 as a 64-bit integer, using integer operations only (the value of a float is
-// mantissa * 2^(exponent - 23), so the product is a shift of the mantissa). Bits below 2^-32
-// are truncated. Summing these integers is exact and independent of the order, which makes the
-// reductions deterministic. |x| >= 2^30, infinities and NaN saturate to +-2^62 (no shift past the
-// word); callers that take terms from outside check the range themselves (fix32_in_range).
+// x * 2^32 as a 64-bit integer, rounded towards zero (bits below 2^-32 are dropped; the scaling is
+// exact). Summing these integers is exact and independent of the order, which makes the reductions
+// deterministic. |x| >= 2^30, infinities and NaN saturate to +-2^62 by their sign; callers that take
+// terms from outside check the range themselves (fix32_in_range).
 __device__ __forceinline__ bool fix32_in_range(float x) { return fabsf(x) < 1073741824.0f; }
 __device__ __forceinline__ long long f32_to_fix32(float x) {
-  const unsigned b = __float_as_uint(x);
-  const int e = (int)((b >> 23) & 0xffu);
-  if (e == 0) return 0;  // zero or subnormal: below the resolution
-  if (e >= 127 + 30) return (b >> 31) ? -(1LL << 62) : (1LL << 62);
-  const long long m = (long long)((b & 0x7fffffu) | 0x800000u);
-  const int sh = e - 127 - 23 + 32;
-  long long v = sh >= 0 ? (m << sh) : (sh > -64 ? (m >> (-sh)) : 0);
-  return (b >> 31) ? -v : v;
+  const long long sat = (__float_as_uint(x) >> 31) ? -(1LL << 62) : (1LL << 62);
+  return fix32_in_range(x) ? __float2ll_rz(x * 4294967296.0f) : sat;
 }
 
 // Warp-wide sum of a 64-bit integer (exact).

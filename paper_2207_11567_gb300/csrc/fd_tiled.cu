@@ -1,7 +1,9 @@
 // Host side of the tiled FD update (fd_tiled.cuh): eligibility, TMA tensor maps, launch.
 #include <algorithm>
 #include <cstdlib>
+#include <cstring>
 #include <new>
+#include <vector>
 #include "fd_tiled.cuh"
 #include "launch.h"
 
@@ -73,31 +75,72 @@ cudaError_t fd_tiled_setup(FDTiledMaps& m, const Geo& g, int K, void* const T[2]
   ok = ok && make_map(&m.U, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, u, g, 3);
   ok = ok && make_map(&m.S, CU_TENSOR_MAP_DATA_TYPE_UINT32, sword, g, 1);
   if (!ok) return cudaErrorInvalidValue;
-  // z chunks: about eleven waves of two resident blocks per SM (the last, partial wave then costs
-  // little; on the 384x192x192 case 12 chunks of 16 planes ran 0.4% faster than 7 of 28, 4 chunks
-  // 2% slower), at least 8 planes per chunk
-  const int gx = (g.nx + TT_X - 1) / TT_X, gy = (g.ny + TT_Y - 1) / TT_Y;
-  int nzc = (11 * 2 * n_sm + gx * gy - 1) / (gx * gy);
-  nzc = std::max(1, std::min(nzc, g.nz / 8));
-  if (const char* s = std::getenv("HLBM_FD_CHUNKS")) nzc = std::max(1, std::min(atoi(s), g.nz));
-  m.lz = (g.nz + nzc - 1) / nzc;
-  m.grid = dim3(gx, gy, (g.nz + m.lz - 1) / m.lz);
+  m.gx = (g.nx + TT_X - 1) / TT_X;
+  m.gy = (g.ny + TT_Y - 1) / TT_Y;
+  m.slots = 2 * n_sm;
   cudaError_t e = set_smem<6, 2>();
   if (e == cudaSuccess) e = set_smem<4, 1>();
   return e;
 }
 
-int fd_tiled_blocks(const FDTiledMaps& m) { return (int)(m.grid.x * m.grid.y * m.grid.z); }
+int fd_tiled_tiles(const FDTiledMaps& m, const Geo& g) { return m.gx * m.gy * ((g.nz + TT_LZ_MIN - 1) / TT_LZ_MIN); }
+
+int fd_tiled_blocks(const FDTiledMaps& m) { return m.n_tiles; }
+
+// The tiles to launch: those with a fluid cell (swirl burner, all tiles / these: 384x192x192, where 22% of
+// the cells are solid, 759 / 698 us per update, 192x96x96 150.2 / 147.5), for the number of planes per
+// tile that costs least: whole waves of the resident blocks (two per SM), each as long as its planes plus
+// about three for the block's start (its first three plane loads and the -z face). Planes per tile, update
+// of 384x192x192: 6 733 us, 8 718, 12 708, 16 709, 24 716; of 192x96x96 with curved walls: 6 166, 8 163.5,
+// 12 162.3, 16 183.8 (one wave and a short second one).
+cudaError_t fd_tiled_set_mask(FDTiledMaps& m, const Geo& g, const uint8_t* mask, int* tiles_dev, cudaStream_t st) {
+  const size_t cols = (size_t)m.gx * m.gy;
+  std::vector<uint8_t> live(cols * g.nz, 0);  // per plane
+  for (int z = 0; z < g.nz; ++z)
+    for (int y = 0; y < g.ny; ++y) {
+      const uint8_t* row = mask + (size_t)g.nx * (y + (size_t)g.ny * z);
+      uint8_t* l = live.data() + cols * z + (size_t)m.gx * (y / TT_Y);
+      for (int t = 0; t < m.gx; ++t)
+        if (!l[t] && std::memchr(row + t * TT_X, 0, std::min(TT_X, g.nx - t * TT_X))) l[t] = 1;
+    }
+  auto tiles_of = [&](int lz) {
+    std::vector<int> list;
+    for (int z0 = 0, k = 0; z0 < g.nz; z0 += lz, ++k)
+      for (size_t t = 0; t < cols; ++t) {
+        bool any = false;
+        for (int z = z0; z < std::min(z0 + lz, g.nz) && !any; ++z) any = live[cols * z + t] != 0;
+        if (any) list.push_back((int)(t + cols * k));
+      }
+    return list;
+  };
+  std::vector<int> list;
+  double best = 1e30;
+  for (int lz = std::min(TT_LZ_MIN, g.nz); lz <= std::min(g.nz, TT_LZ_MAX); ++lz) {
+    std::vector<int> l = tiles_of(lz);
+    const double cost = (double)(((int)l.size() + m.slots - 1) / m.slots) * (lz + 3);
+    if (cost < best) {
+      best = cost;
+      m.lz = lz;
+      list.swap(l);
+    }
+  }
+  m.tiles = tiles_dev;
+  m.n_tiles = (int)list.size();
+  if (list.empty()) return cudaSuccess;
+  const cudaError_t e = cudaMemcpyAsync(tiles_dev, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
 
 cudaError_t launch_fd_tiled(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st) {
+  if (m.n_tiles == 0) return cudaSuccess;
   const dim3 block(TT_X, TT_Y);
   const int sensor = a.Floc ? 1 : 0;
   if (a.c.K == 6 && a.c.nrx == 2)
-    fd_tiled_kernel<6, 2><<<m.grid, block, TTLayout<6>::BYTES, st>>>(a, m.T[cur], m.Y[cur], m.U, m.F[cur], m.S,
-                                                                      m.lz, sensor);
+    fd_tiled_kernel<6, 2><<<m.n_tiles, block, TTLayout<6>::BYTES, st>>>(a, m.T[cur], m.Y[cur], m.U, m.F[cur], m.S,
+                                                                         m.tiles, m.lz, sensor);
   else
-    fd_tiled_kernel<4, 1><<<m.grid, block, TTLayout<4>::BYTES, st>>>(a, m.T[cur], m.Y[cur], m.U, m.F[cur], m.S,
-                                                                      m.lz, sensor);
+    fd_tiled_kernel<4, 1><<<m.n_tiles, block, TTLayout<4>::BYTES, st>>>(a, m.T[cur], m.Y[cur], m.U, m.F[cur], m.S,
+                                                                         m.tiles, m.lz, sensor);
   return cudaGetLastError();
 }
 

@@ -27,12 +27,21 @@
 //   the cell it copies), so that every field reads its face values with four plain loads; the
 //   z face selects among its four register values.
 //
+// * Two fields of a pair go through each instruction of a face (packed.cuh); a block is launched only for
+//   a tile that holds fluid, and a row of cells without a fluid face skips the face work.
+//
+// Bound by instruction issue (58% of the issue slots, the rest waits on barriers, shared memory and the
+// chain of each face), not by memory: swirl burner 384x192x192, FP32, 10.97 M fluid cells, 808 us per
+// update with one field per instruction and all tiles, 698 us so (126 us of traffic at the copy rate).
+// Packed faces, reciprocals and conversions: 808 -> 765 us; rows without fluid 759; tile list 698.
+//
 // Cells flagged with ghost-point wall weights (SW_WALL) are left to fd_step_kernel (walls-only
 // launch); the tiled kernel needs non-periodic faces and nx a multiple of 4 (TMA strides).
 #pragma once
 #include <cuda.h>
 #include <type_traits>
 #include "fd_kernel.cuh"
+#include "packed.cuh"
 
 namespace hlbm {
 
@@ -42,6 +51,7 @@ constexpr int TT_PX = TT_X + 2 * TT_HX;     // 40
 constexpr int TT_PY = TT_Y + 2 * TT_HY;     // 12
 constexpr int TT_PLANE = TT_PX * TT_PY;     // 480 words per plane array
 constexpr int TT_SLOTS = 4;
+constexpr int TT_LZ_MIN = 4, TT_LZ_MAX = 16;  // planes per tile
 constexpr int TT_FX = TT_X + 2, TT_FY = TT_Y + 2;  // F mu tile, halo 1
 // planes of one slot: T, Y_0..Y_{K-1}, u_x, u_y, u_z, F_loc, stencil word
 template <int NK> struct TTLayout {
@@ -61,7 +71,10 @@ template <int NK> struct TTLayout {
 struct FDTiledMaps {
   CUtensorMap T[2], Y[2], F[2], U, S;
   int lz = 0;              // planes per block along z
-  dim3 grid;
+  int gx = 0, gy = 0;      // tiles of a plane
+  int slots = 0;           // resident blocks of the GPU
+  int* tiles = nullptr;    // [n_tiles] the tiles that hold fluid: x + gx (y + gy z)
+  int n_tiles = 0;
   bool sensor = false;
 };
 
@@ -188,21 +201,26 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, u
 
 constexpr int TT_THREADS = TT_X * TT_Y;
 
-// WENO3 face value and diffusive flux (without the field's 1/(Pr Le)) from the four stencil values
-// (a - e, a, b, b + e) of the face between a and b = a + e, ghosts already substituted. Same
+// WENO3 face values of two fields and their differences d across the face, from the four stencil
+// values (a - e, a, b, b + e) of the face between a and b = a + e, ghosts already substituted. Same
 // formulas as fd_cell: with d1 = v0 - vm, d2 = v1 - v0, d3 = v2 - v1 and t(d) = (eps + d^2)^2, the
 // face is v0 + (t(d2) d1 + 2 t(d1) d2) / (2 (t(d2) + 2 t(d1))) upwind from a, and
-// v1 - (t(d2) d3 + 2 t(d3) d2) / (2 (t(d2) + 2 t(d3))) upwind from b.
-__device__ __forceinline__ void face_math(float vm, float v0, float v1, float v2, bool up, float FMf, float eps,
-                                          float& Fv, float& Dv) {
-  const float d1 = v0 - vm, d2 = v1 - v0, d3 = v2 - v1;
-  const float s = up ? d1 : d3;
-  const float ss = fmaf(s, s, eps), s2 = fmaf(d2, d2, eps);
-  const float ts = ss * ss, t2 = s2 * s2;
-  const float num = fmaf(t2, s, 2.0f * ts * d2);
-  const float q = num * rcp_approx(fmaf(2.0f, ts, t2));
-  Fv = up ? fmaf(0.5f, q, v0) : fmaf(-0.5f, q, v1);
-  Dv = FMf * d2;
+// v1 - (t(d2) d3 + 2 t(d3) d2) / (2 (t(d2) + 2 t(d3))) upwind from b. The diffusive flux (without the
+// field's 1/(Pr Le)) is 0.5 (F mu (a) + F mu (b)) d. Two fields go through each instruction
+// (packed.cuh); every field is rounded as by the scalar form.
+__device__ __forceinline__ void face_math2(F2 vm, F2 v0, F2 v1, F2 v2, bool up, float h, F2 eps, F2& Fv, F2& d) {
+  const F2 two = splat<F2>(2.0);
+  const F2 d1 = v0 - vm, d3 = v2 - v1;
+  d = v1 - v0;
+  F2 s, b;
+  s.v = up ? d1.v : d3.v;
+  b.v = up ? v0.v : v1.v;
+  const F2 ss = fma_(s, s, eps), s2 = fma_(d, d, eps);
+  const F2 ts = ss * ss, t2 = s2 * s2;
+  const F2 num = fma_(t2, s, (two * ts) * d);
+  const F2 den = fma_(two, ts, t2);
+  const F2 q = num * pack2(rcp_approx(lo(den)), rcp_approx(hi(den)));
+  Fv = fma_(pack2(h, h), q, b);
 }
 
 // A face of the plane tile: the plane indices of its four stencil values after ghost
@@ -210,7 +228,7 @@ __device__ __forceinline__ void face_math(float vm, float v0, float v1, float v2
 struct TFace {
   int im, i0, i1, i2;
   bool up;
-  float FMf;
+  float FMf, h;  // h = up ? 1/2 : -1/2
 };
 
 // Face between tile points ia and ia + st (plane indices; st = 1 along x, TT_PX along y), from the
@@ -255,14 +273,37 @@ __device__ __forceinline__ TFace tile_face(const float* __restrict__ sS, const f
   f.i2 = ia + o2 * st;
   f.FMf = 0.5f * (FMown + FMn);
   f.up = 0.5f * (uown + un) >= 0.0f;
+  f.h = f.up ? 0.5f : -0.5f;
   return f;
+}
+
+// reaction_rates with the species of each order read from the plane tile by its index (Yp: species 0 of
+// this cell) instead of picked out of registers by selects.
+template <int NR>
+__device__ __forceinline__ void tile_rates(const FDConst<float>& c, float T, float inv_T, const float* __restrict__ Yp,
+                                           float rho_phys, float* q) {
+#pragma unroll
+  for (int j = 0; j < NR; ++j) {
+    float v = c.A[j] * arrhenius(c.ER_hi[j], c.ER_lo[j], T, inv_T);
+    if (c.beta[j] != 0.0f) v *= powr<float>(T, c.beta[j]);
+#pragma unroll
+    for (int m = 0; m < MAX_ORD; ++m) {
+      if (m >= c.nord[j]) break;
+      const int k = c.ord_k[j][m];
+      const float n = c.ord_n[j][m];
+      const float conc = rho_phys * fmaxf(Yp[k * TT_PLANE], 0.0f) * c.inv_W[k];
+      v *= (n == 1.0f) ? conc : powr<float>(conc, n);
+    }
+    q[j] = v;
+  }
 }
 
 template <int NK, int NR>
 __global__ void __launch_bounds__(TT_THREADS, 2)
     fd_tiled_kernel(const FDArgs<float> a, const __grid_constant__ CUtensorMap mT, const __grid_constant__ CUtensorMap mY,
                     const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUtensorMap mF,
-                    const __grid_constant__ CUtensorMap mS, const int LZ, const int sensor) {
+                    const __grid_constant__ CUtensorMap mS, const int* __restrict__ tiles, const int LZ,
+                    const int sensor) {
   using L = TTLayout<NK>;
   extern __shared__ __align__(128) float sm[];
   float* ring = sm;
@@ -276,7 +317,9 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
   const Geo& g = a.geo;
   const int nx = g.nx, ny = g.ny, nz = g.nz, N = g.N;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + TT_X * ty;
-  const int x0 = blockIdx.x * TT_X, y0 = blockIdx.y * TT_Y, z0 = blockIdx.z * LZ;
+  const int tile = __ldg(tiles + blockIdx.x);
+  const int gx = (nx + TT_X - 1) / TT_X, gy = (ny + TT_Y - 1) / TT_Y, trow = tile / gx;
+  const int x0 = (tile - trow * gx) * TT_X, y0 = (trow % gy) * TT_Y, z0 = (trow / gy) * LZ;
   const int z1 = min(z0 + LZ, nz);
   const int x = x0 + tx, y = y0 + ty;
   const bool in_xy = x < nx && y < ny;
@@ -448,16 +491,16 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
     for (int j = 0; j < NR; ++j) q[j] = 0.0f;
     float inv_T = 0.0f;
     if (active) {
-      // one IEEE reciprocal each of T, sum Y/W and rho, reused where fd_cell divides
-      inv_T = 1.0f / Tr;
-      W = 1.0f / sW;
+      // one reciprocal (rounded as the IEEE one) each of T, sum Y/W and rho, reused where fd_cell divides
+      inv_T = rcp_(Tr);
+      W = rcp_(sW);
       rho = fdr * W * inv_T;
       const float rho_phys = rho * c.rho_ref_f;
-      inv_rho = 1.0f / rho;
-      reaction_rates<NR, float, NK>(c, Tr, inv_T, Yr, rho_phys, q);
+      inv_rho = rcp_(rho);
+      tile_rates<NR>(c, Tr, inv_T, s0 + L::P_Y * TT_PLANE + own, rho_phys, q);
 #pragma unroll
       for (int j = 0; j < NR; ++j) qdot += c.heat[j] * q[j];
-      inv_rpF = inv_rho * c.inv_rho_ref / Fr;
+      inv_rpF = div_(inv_rho * c.inv_rho_ref, Fr, rcp_(Fr));
     }
 
     // ---- faces of this plane: +x, +y of this cell as source indices, +z as selects; the
@@ -469,9 +512,11 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
     TFace fx, fy;
     if (plain) {
       fx = {own - 1, own, own + 1, own + 2, 0.5f * (ux + s0[L::P_U * TT_PLANE + own + 1]) >= 0.0f,
-            0.5f * (FMs[fo] + FMs[fo + 1])};
+            0.5f * (FMs[fo] + FMs[fo + 1]), 0.0f};
       fy = {own - TT_PX, own, own + TT_PX, own + 2 * TT_PX,
-            0.5f * (uy + s0[(L::P_U + 1) * TT_PLANE + own + TT_PX]) >= 0.0f, 0.5f * (FMs[fo] + FMs[fo + TT_FX])};
+            0.5f * (uy + s0[(L::P_U + 1) * TT_PLANE + own + TT_PX]) >= 0.0f, 0.5f * (FMs[fo] + FMs[fo + TT_FX]), 0.0f};
+      fx.h = fx.up ? 0.5f : -0.5f;
+      fy.h = fy.up ? 0.5f : -0.5f;
     } else {
       fx = tile_face(sS, s0 + L::P_U * TT_PLANE, FMs, own, 1, fo, 1, 0);
       fy = tile_face(sS, s0 + (L::P_U + 1) * TT_PLANE, FMs, own, TT_PX, fo, TT_FX, 1);
@@ -521,39 +566,76 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
       FMz = 0.5f * (FMown + FMn);
       upz = 0.5f * (uown + un) >= 0.0f;
     }
+    const float hz = upz ? 0.5f : -0.5f;
+    const bool zghost = __any_sync(0xffffffffu, zcm || zc0 || zc1 || zc2);
+
+    // a row of cells that neither is fluid nor shares a +x, +y or +z face with fluid does no face work
+    const bool live = __any_sync(0xffffffffu, ((sw | __float_as_uint(sS[own + 1]) | __float_as_uint(sS[own + TT_PX]) |
+                                               (z + 1 < nz ? __float_as_uint(s1[L::P_S * TT_PLANE + own]) : 0u)) >> 31) != 0u);
 
     // ---- fields: 0 = T, 1.. = Y_k, in pairs (one barrier per pair)
     float lam = 0.0f, sWn = 0.0f, Tnew = Tr, yf_new = 0.0f, yo_new = 0.0f;
 #pragma unroll
     for (int p = 0; p <= NK; p += 2) {
       float Fxp[2], Dxp[2], Fyp[2], Dyp[2], Fzp[2], Dzp[2];
-      const int pb = (p >> 1) & 1;  // face buffers of this pair: 2 pb, 2 pb + 1
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int fi = p + h;
-        if (fi > NK) break;
-        const float* P = s0 + (L::P_T + fi) * TT_PLANE;
-        const float eps = fi == 0 ? c.eps_T : c.eps_Y;
-        float2* xf = XF + (2 * pb + h) * TT_Y * (TT_X + 1);
-        float2* yf = YF + (2 * pb + h) * (TT_Y + 1) * TT_X;
-        const float pr = P[own];
-        face_math(P[fx.im], P[fx.i0], P[fx.i1], P[fx.i2], fx.up, fx.FMf, eps, Fxp[h], Dxp[h]);
-        face_math(P[fy.im], P[fy.i0], P[fy.i1], P[fy.i2], fy.up, fy.FMf, eps, Fyp[h], Dyp[h]);
+      const int pb = (p >> 1) & 1;       // face buffers of this pair: 2 pb, 2 pb + 1
+      const int p1 = p < NK ? p + 1 : p;  // the last field of an odd count goes twice
+      const float* P0 = s0 + (L::P_T + p) * TT_PLANE;
+      const float* P1 = s0 + (L::P_T + p1) * TT_PLANE;
+      const F2 eps = pack2(p == 0 ? c.eps_T : c.eps_Y, c.eps_Y);
+      float2* xf = XF + 2 * pb * TT_Y * (TT_X + 1);
+      float2* yf = YF + 2 * pb * (TT_Y + 1) * TT_X;
+      constexpr int XS = TT_Y * (TT_X + 1), YS = (TT_Y + 1) * TT_X;
+      if (live) {
+        F2 F, d;
+        face_math2(pack2(P0[fx.im], P1[fx.im]), pack2(P0[fx.i0], P1[fx.i0]), pack2(P0[fx.i1], P1[fx.i1]),
+                   pack2(P0[fx.i2], P1[fx.i2]), fx.up, fx.h, eps, F, d);
+        Fxp[0] = lo(F);
+        Fxp[1] = hi(F);
+        Dxp[0] = fx.FMf * lo(d);
+        Dxp[1] = fx.FMf * hi(d);
+        face_math2(pack2(P0[fy.im], P1[fy.im]), pack2(P0[fy.i0], P1[fy.i0]), pack2(P0[fy.i1], P1[fy.i1]),
+                   pack2(P0[fy.i2], P1[fy.i2]), fy.up, fy.h, eps, F, d);
+        Fyp[0] = lo(F);
+        Fyp[1] = hi(F);
+        Dyp[0] = fy.FMf * lo(d);
+        Dyp[1] = fy.FMf * hi(d);
         {
-          const float v1r = s1[(L::P_T + fi) * TT_PLANE + own], v2r = s2[(L::P_T + fi) * TT_PLANE + own];
-          const float v0 = zc0 ? v1r : pr;
-          const float v1 = zc1 ? pr : v1r;
-          const float vm = zcm ? v0 : phim[fi];
-          const float v2 = zc2 ? v1 : v2r;
-          face_math(vm, v0, v1, v2, upz, FMz, eps, Fzp[h], Dzp[h]);
+          const float* Q0 = s1 + (L::P_T + p) * TT_PLANE + own;
+          const float* Q1 = s1 + (L::P_T + p1) * TT_PLANE + own;
+          const F2 pr = pack2(P0[own], P1[own]), v1r = pack2(*Q0, *Q1);
+          const F2 v2r = pack2(s2[(L::P_T + p) * TT_PLANE + own], s2[(L::P_T + p1) * TT_PLANE + own]);
+          F2 v0 = pr, v1 = v1r, vm = pack2(phim[p], phim[p1]), v2 = v2r;
+          if (zghost) {
+            v0.v = zc0 ? v1r.v : pr.v;
+            v1.v = zc1 ? pr.v : v1r.v;
+            vm.v = zcm ? v0.v : vm.v;
+            v2.v = zc2 ? v1.v : v2r.v;
+          }
+          face_math2(vm, v0, v1, v2, upz, hz, eps, F, d);
+          Fzp[0] = lo(F);
+          Fzp[1] = hi(F);
+          Dzp[0] = FMz * lo(d);
+          Dzp[1] = FMz * hi(d);
         }
-        xf[ty * (TT_X + 1) + tx + 1] = make_float2(Fxp[h], Dxp[h]);
-        yf[(ty + 1) * TT_X + tx] = make_float2(Fyp[h], Dyp[h]);
-        if (edge_y || edge_x) {
-          float Fe, De;
-          face_math(P[fe.im], P[fe.i0], P[fe.i1], P[fe.i2], fe.up, fe.FMf, eps, Fe, De);
-          if (edge_y) yf[tx] = make_float2(Fe, De);
-          else xf[tx * (TT_X + 1)] = make_float2(Fe, De);
+        xf[ty * (TT_X + 1) + tx + 1] = make_float2(Fxp[0], Dxp[0]);
+        yf[(ty + 1) * TT_X + tx] = make_float2(Fyp[0], Dyp[0]);
+        if (p < NK) {
+          xf[XS + ty * (TT_X + 1) + tx + 1] = make_float2(Fxp[1], Dxp[1]);
+          yf[YS + (ty + 1) * TT_X + tx] = make_float2(Fyp[1], Dyp[1]);
+        }
+      }
+      if (edge_y || edge_x) {
+        F2 F, d;
+        face_math2(pack2(P0[fe.im], P1[fe.im]), pack2(P0[fe.i0], P1[fe.i0]), pack2(P0[fe.i1], P1[fe.i1]),
+                   pack2(P0[fe.i2], P1[fe.i2]), fe.up, fe.h, eps, F, d);
+        const float2 e0 = make_float2(lo(F), fe.FMf * lo(d)), e1 = make_float2(hi(F), fe.FMf * hi(d));
+        if (edge_y) {
+          yf[tx] = e0;
+          if (p < NK) yf[YS + tx] = e1;
+        } else {
+          xf[tx * (TT_X + 1)] = e0;
+          if (p < NK) xf[XS + tx * (TT_X + 1)] = e1;
         }
       }
       __syncthreads();
@@ -561,6 +643,7 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
       for (int h = 0; h < 2; ++h) {
         const int fi = p + h;
         if (fi > NK) break;
+        if (!live) continue;
         const float pr = s0[(L::P_T + fi) * TT_PLANE + own];
         const float2 xm = XF[(2 * pb + h) * TT_Y * (TT_X + 1) + ty * (TT_X + 1) + tx];
         const float2 ym = YF[(2 * pb + h) * (TT_Y + 1) * TT_X + ty * TT_X + tx];
@@ -568,7 +651,6 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
         carF[fi] = Fzp[h];
         carD[fi] = Dzp[h];
         phim[fi] = pr;
-        if (!active) continue;
         const float adv = ux * (Fxp[h] - xm.x) + uy * (Fyp[h] - ym.x) + uz * (Fzp[h] - Fzm);
         float dif = (Dxp[h] - xm.y) + (Dyp[h] - ym.y) + (Dzp[h] - Dzm);
         const float gfac = c.inv_Pr * (fi == 0 ? 1.0f : c.inv_Le[fi - 1]);
@@ -585,11 +667,11 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
         const float NA = dif + src;
         const float pn = pr - adv + NA;
         if (fi == 0) {
-          a.T_out[r] = pn;
+          if (active) a.T_out[r] = pn;
           lam += NA * inv_T;
           Tnew = pn;
         } else {
-          a.Y_out[(size_t)(fi - 1) * N + r] = pn;
+          if (active) a.Y_out[(size_t)(fi - 1) * N + r] = pn;
           lam += W * c.inv_W[fi - 1] * NA;
           sWn += pn * c.inv_W[fi - 1];
           if (fi - 1 == c.sensor_species) yf_new = pn;
@@ -598,11 +680,17 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
       }
     }
     if (active) {
-      if (a.Floc_out) a.Floc_out[r] = sensor_floc<float>(c, Tnew, yf_new, yo_new);
+      if (a.Floc_out) {  // sensor_floc
+        const float om = fmaxf(yf_new, 0.0f) * fmaxf(yo_new, 0.0f) * expf(div_(-c.sensor_Ta, Tnew, rcp_(Tnew)));
+        a.Floc_out[r] = 1.0f + (c.F - 1.0f) * tanhf(c.sensor_beta * om * c.inv_wref);
+      }
       a.rho_out[r] = rho;
       a.lam_out[r] = lam;
       if (c.closed) {
-        accI += f32_to_fix32(c.I_scale / (sWn * Tnew));
+        {
+          const float wt = sWn * Tnew;
+          accI += f32_to_fix32(div_(c.I_scale, wt, rcp_(wt)));
+        }
         if (x == 0 && g.bc_lo[0] == BC_INLET) accM += f32_to_fix32(c.M_scale * rin * __ldg(a.inlet_u + y + ny * z));
         if (x == nx - 1 && g.bc_hi[0] == BC_OUTLET) accM += f32_to_fix32(-(c.M_scale * rho * ux));
       }
@@ -623,10 +711,9 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
       tI += red[2 * w];
       tM += red[2 * w + 1];
     }
-    const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     long long* out = (long long*)a.partials;
-    out[2 * bid] = tI;
-    out[2 * bid + 1] = tM;
+    out[2 * blockIdx.x] = tI;
+    out[2 * blockIdx.x + 1] = tM;
   }
 }
 

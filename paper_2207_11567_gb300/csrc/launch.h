@@ -20,7 +20,10 @@ void fd_tiled_destroy(FDTiledMaps* m);
 // T, Y, F: the two state parities (F nullptr without the flame sensor); n_sm: SMs of the device
 cudaError_t fd_tiled_setup(FDTiledMaps& m, const Geo& g, int K, void* const T[2], void* const Y[2],
                            void* const F[2], const void* u, const uint32_t* sword, int n_sm);
-int fd_tiled_blocks(const FDTiledMaps& m);
+int fd_tiled_tiles(const FDTiledMaps& m, const Geo& g);  // at most
+int fd_tiled_blocks(const FDTiledMaps& m);  // that hold fluid (blocks of a launch, partial slots)
+// the tiles to launch, from the host copy of the mask; tiles_dev: device array of fd_tiled_tiles ints
+cudaError_t fd_tiled_set_mask(FDTiledMaps& m, const Geo& g, const uint8_t* mask, int* tiles_dev, cudaStream_t st);
 cudaError_t launch_fd_tiled(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st);
 
 // fd_split.cu: FD update of small 2-D FP64 grids, one warp per field (no options, no wall weights)
