@@ -515,6 +515,9 @@ __global__ void __launch_bounds__(FD_BLOCK, sizeof(R) == 4 ? MINB : 1)
   int x, y, z, r;
   bool inside;
   if (a.wall_list) {
+    // the tiled update of the other cells may start: it writes none of what this launch reads, and what both
+    // read is complete (this launch waited for its predecessors before its first block)
+    pdl_trigger();
     // one thread per listed cell (a 1-D grid of blocks of the same shape)
     const int wrow = blockIdx.x * FD_BLOCK + threadIdx.x + FDShape<D>::X * (threadIdx.y + FDShape<D>::Y * threadIdx.z);
     inside = wrow < a.n_wall_list;
@@ -530,7 +533,7 @@ __global__ void __launch_bounds__(FD_BLOCK, sizeof(R) == 4 ? MINB : 1)
     r = x + g.nx * (y + g.ny * z);
   }
   const uint32_t sw = inside ? __ldg(a.sword + r) : 0u;
-  // walls_only: the launch after the tiled update, for the cells with ghost-point wall weights
+  // walls_only: the launch beside the tiled update, for the cells with ghost-point wall weights
   const bool active = (sw >> 31) != 0u && (!a.walls_only || (sw & SW_WALL) != 0u);
   R termI = R(0), termM = R(0);  // P_th integrand and boundary mass flux of this cell
 

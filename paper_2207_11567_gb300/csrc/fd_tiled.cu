@@ -131,17 +131,27 @@ cudaError_t fd_tiled_set_mask(FDTiledMaps& m, const Geo& g, const uint8_t* mask,
   return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
 }
 
-cudaError_t launch_fd_tiled(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st) {
+namespace {
+template <int NK, int NR>
+cudaError_t launch_tiles(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st, bool pdl) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(m.n_tiles);
+  cfg.blockDim = dim3(TT_X, TT_Y);
+  cfg.dynamicSmemBytes = TTLayout<NK>::BYTES;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fd_tiled_kernel<NK, NR>, a, m.T[cur], m.Y[cur], m.U, m.F[cur], m.S,
+                            (const int*)m.tiles, m.lz, a.Floc ? 1 : 0);
+}
+}  // namespace
+
+cudaError_t launch_fd_tiled(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st, bool pdl) {
   if (m.n_tiles == 0) return cudaSuccess;
-  const dim3 block(TT_X, TT_Y);
-  const int sensor = a.Floc ? 1 : 0;
-  if (a.c.K == 6 && a.c.nrx == 2)
-    fd_tiled_kernel<6, 2><<<m.n_tiles, block, TTLayout<6>::BYTES, st>>>(a, m.T[cur], m.Y[cur], m.U, m.F[cur], m.S,
-                                                                         m.tiles, m.lz, sensor);
-  else
-    fd_tiled_kernel<4, 1><<<m.n_tiles, block, TTLayout<4>::BYTES, st>>>(a, m.T[cur], m.Y[cur], m.U, m.F[cur], m.S,
-                                                                         m.tiles, m.lz, sensor);
-  return cudaGetLastError();
+  return a.c.K == 6 && a.c.nrx == 2 ? launch_tiles<6, 2>(a, m, cur, st, pdl) : launch_tiles<4, 1>(a, m, cur, st, pdl);
 }
 
 }  // namespace hlbm

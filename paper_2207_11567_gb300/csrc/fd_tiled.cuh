@@ -35,8 +35,9 @@
 // update with one field per instruction and all tiles, 698 us so (126 us of traffic at the copy rate).
 // Packed faces, reciprocals and conversions: 808 -> 765 us; rows without fluid 759; tile list 698.
 //
-// Cells flagged with ghost-point wall weights (SW_WALL) are left to fd_step_kernel (walls-only
-// launch); the tiled kernel needs non-periodic faces and nx a multiple of 4 (TMA strides).
+// Cells flagged with ghost-point wall weights (SW_WALL) are left to fd_step_kernel (walls-only launch
+// just before this kernel, which starts beside it); the tiled kernel needs non-periodic faces and nx a
+// multiple of 4 (TMA strides).
 #pragma once
 #include <cuda.h>
 #include <type_traits>
@@ -402,6 +403,7 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
   if (!ok) {
     if (tid == 0) atomicOr(a.flag, 4);
     for (int zp = z0; zp <= min(z0 + 2, zlast); ++zp) wait(zp);
+    pdl_wait();
     return;
   }
   // ghosts and F mu tile of plane z0 (each step of the march prepares the plane above it)
@@ -462,6 +464,7 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
     if (!__syncthreads_and(okz)) {
       if (tid == 0) atomicOr(a.flag, 4);
       for (int zp = z; zp <= min(z + 3, zlast); ++zp) wait(zp);
+      pdl_wait();
       return;
     }
     if (tid == 0 && z + 3 <= zlast) {
@@ -696,6 +699,9 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
       }
     }
   }
+
+  // with wall cells: their launch, which this one may have overtaken, completes before this one does
+  pdl_wait();
 
   // ---------------------------------------------------------------- P_th partial of this block
   if (!c.closed) return;

@@ -24,7 +24,8 @@ int fd_tiled_tiles(const FDTiledMaps& m, const Geo& g);  // at most
 int fd_tiled_blocks(const FDTiledMaps& m);  // that hold fluid (blocks of a launch, partial slots)
 // the tiles to launch, from the host copy of the mask; tiles_dev: device array of fd_tiled_tiles ints
 cudaError_t fd_tiled_set_mask(FDTiledMaps& m, const Geo& g, const uint8_t* mask, int* tiles_dev, cudaStream_t st);
-cudaError_t launch_fd_tiled(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st);
+// pdl: the launch before it (wall cells) has triggered its dependents; the two run side by side
+cudaError_t launch_fd_tiled(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st, bool pdl);
 
 // fd_split.cu: FD update of small 2-D FP64 grids, one warp per field (no options, no wall weights)
 constexpr int FD_SPLIT_MAX = 32768;
