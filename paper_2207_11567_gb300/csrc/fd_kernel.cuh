@@ -188,7 +188,7 @@ template <int DEG, typename R> __device__ __forceinline__ R hW_eval(const R (&a)
 // the arithmetic means G_k,f, Y_k,f and dlnW = (W_n - W_r) / mean W, the species term is
 //   sum_faces [G_k,f (dY_k + Y_k,f dlnW) - Y_k,f C_f],  C_f = sum_j G_j,f (dY_j + Y_j,f dlnW)
 // (differences neighbour minus cell), the Hirschfelder-Curtiss flux with its correction velocity.
-template <int D, typename R, int NK, int NR, bool FAST, int VDEG, bool GW = false, bool MIX = false>
+template <int D, typename R, int NK, int NR, bool FAST, int VDEG, bool GW = false, bool MIX = false, int FU = 1>
 __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z, int r, uint32_t sw, R& termI,
                                         R& termM) {
   const FDConst<R>& c = a.c;
@@ -376,7 +376,7 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
       }
     }
     // fields: 0 = T, 1.. = Y_k (VCP: the species first, T last)
-#pragma unroll 1
+#pragma unroll FU
     for (int it = 0; it <= K; ++it) {
       const int fi = VCP ? (it == K ? 0 : it + 1) : it;
       R ckr = R(0);
@@ -506,10 +506,19 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
 
 // NK, NR > 0: species and reaction counts known at compile time (loops unroll exactly);
 // NK = NR = 0: counts read from the constants at run time.
-// MINB: FP32 resident blocks per SM that the register budget is sized for.
+// MINB: FP32 resident blocks per SM that the register budget is sized for. FD_UNROLLED (constant heat
+// capacities): the loop over the fields is unrolled as well, so that the loads of later fields are in flight
+// while one is computed. In 2-D the update is a chain of latencies at most sizes (512x128 cells: 14 of 64
+// warps per SM) and bound by issue at the largest; 6 species, step of chamber / flame, fields rolled at
+// 4 blocks / unrolled at 3: 256x1 (4 species) 9.5 / 8.5 us, 128x64 12.5 / 10.4, 512x128 14.6 / 12.5, 600x160 16.6 / 14.5,
+// 512x256 18.6 / 17.4, 1024x256 25.8 / 23.7, 2048x512 82.3 / 77.3; unrolled at 2 blocks 15.6 at 600x160, 24.9 at
+// 1024x256, 90.0 at 2048x512. In 3-D more fields in flight cost more registers than they hide (vessel
+// 135x101x77: two per pass 124 us, rolled 117).
+constexpr int FD_UNROLLED = 3;
 template <int D, typename R, int NK, int NR, int VDEG = 0, bool MIX = false, int MINB = 4>
 __global__ void __launch_bounds__(FD_BLOCK, sizeof(R) == 4 ? MINB : 1)
     fd_step_kernel(const FDArgs<R> a) {
+  constexpr int FU = VDEG == 0 && MINB == FD_UNROLLED ? NK + 1 : 1;
   const FDConst<R>& c = a.c;
   const Geo& g = a.geo;
   int x, y, z, r;
@@ -552,9 +561,9 @@ __global__ void __launch_bounds__(FD_BLOCK, sizeof(R) == 4 ? MINB : 1)
       if (warp_fast) fd_cell<D, R, NK, NR, true, 0, false, true>(a, x, y, z, r, sw, termI, termM);
       else fd_cell<D, R, NK, NR, false, 0, false, true>(a, x, y, z, r, sw, termI, termM);
     } else {
-      if (warp_fast) fd_cell<D, R, NK, NR, true, VDEG>(a, x, y, z, r, sw, termI, termM);
+      if (warp_fast) fd_cell<D, R, NK, NR, true, VDEG, false, false, FU>(a, x, y, z, r, sw, termI, termM);
       else if (warp_walls) fd_cell<D, R, NK, NR, false, VDEG, true>(a, x, y, z, r, sw, termI, termM);
-      else fd_cell<D, R, NK, NR, false, VDEG>(a, x, y, z, r, sw, termI, termM);
+      else fd_cell<D, R, NK, NR, false, VDEG, false, false, FU>(a, x, y, z, r, sw, termI, termM);
     }
   }
   if (!c.closed) return;  // uniform across the grid
@@ -619,8 +628,10 @@ cudaError_t launch_fd(const FDArgs<R>& a, cudaStream_t st, bool sensor_pass) {
   } else {
     const dim3 grid = a.wall_list ? dim3((a.n_wall_list + FD_BLOCK - 1) / FD_BLOCK) : fd_grid<D>(a.geo);
     const dim3 block(FDShape<D>::X, FDShape<D>::Y, FDShape<D>::Z);
-    if (a.c.K == 6 && a.c.nrx == 2) fd_step_kernel<D, R, 6, 2><<<grid, block, 0, st>>>(a);
-    else if (a.c.K == 4 && a.c.nrx == 1) fd_step_kernel<D, R, 4, 1><<<grid, block, 0, st>>>(a);
+    // FP32 in 2-D: the fields unrolled (see fd_step_kernel) with 3 resident blocks
+    constexpr int MINB = D == 2 && sizeof(R) == 4 ? FD_UNROLLED : 4;
+    if (a.c.K == 6 && a.c.nrx == 2) fd_step_kernel<D, R, 6, 2, 0, false, MINB><<<grid, block, 0, st>>>(a);
+    else if (a.c.K == 4 && a.c.nrx == 1) fd_step_kernel<D, R, 4, 1, 0, false, MINB><<<grid, block, 0, st>>>(a);
     else fd_step_kernel<D, R, 0, 0><<<grid, block, 0, st>>>(a);
   }
   return cudaGetLastError();
