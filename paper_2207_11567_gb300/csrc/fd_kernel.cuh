@@ -19,6 +19,7 @@
 // needed only after the state was set from outside.
 #pragma once
 #include "common.cuh"
+#include "packed.cuh"
 
 namespace hlbm {
 
@@ -79,6 +80,14 @@ template <> __device__ __forceinline__ double powr<double>(double x, double y) {
 template <typename R> __device__ __forceinline__ R fdiv(R a, R b) { return a / b; }
 template <> __device__ __forceinline__ float fdiv<float>(float a, float b) { return a * rcp_approx(b); }
 
+// 1 / x and a / b with rb = recip(b): FP32 by a Newton step, rounded as the IEEE operations in the normal
+// range (packed.cuh) without their branches for the rest (FD update, IEEE / these: vessel 135x101x77 117.2 /
+// 114.2 us, swirl 192x96x96 with variable heat capacities 237 / 223, chamber 1024x256 21.2 / 20.5).
+__device__ __forceinline__ float recip(float x) { return rcp_(x); }
+__device__ __forceinline__ float quot(float a, float b, float rb) { return div_(a, b, rb); }
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+__device__ __forceinline__ double quot(double a, double b, double) { return a / b; }
+
 template <typename R> __device__ __forceinline__ R weno3(R a, R b, R c, R eps) {
   const R q0 = R(-0.5) * a + R(1.5) * b;
   const R q1 = R(0.5) * (b + c);
@@ -136,7 +145,7 @@ template <typename R> __device__ __forceinline__ R nu_of(const FDConst<R>& c, in
 // Flame sensor: F_loc = 1 + (F - 1) tanh(beta Omega / Omega_0) with
 // Omega = max(Y_F, 0) max(Y_O, 0) exp(-T_s / T), a function of the cell's own state.
 template <typename R> __device__ __forceinline__ R sensor_floc(const FDConst<R>& c, R T, R yf, R yo) {
-  const R om = fmax(yf, R(0)) * fmax(yo, R(0)) * exp(-c.sensor_Ta / T);
+  const R om = fmax(yf, R(0)) * fmax(yo, R(0)) * exp(quot(-c.sensor_Ta, T, recip(T)));
   return R(1) + (c.F - R(1)) * tanh(c.sensor_beta * om * c.inv_wref);
 }
 
@@ -259,13 +268,13 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
         Yr[k] = R(0);
       }
     }
-    const R W = R(1) / sW;
+    const R W = recip(sW), inv_T = recip(Tr);
     const R fdr = sizeof(R) == 4 ? (R)a.pth->fd_rho : (R)a.pth->fd_rho_d;
-    const R rho = fdr * W / Tr;  // lattice units
-    const R rho_phys = rho / c.inv_rho_ref;
-    const R inv_rho = R(1) / rho;
+    const R rho = quot(fdr * W, Tr, inv_T);  // lattice units
+    const R rho_phys = quot(rho, c.inv_rho_ref, recip(c.inv_rho_ref));
+    const R inv_rho = recip(rho);
     R q[RMAX];
-    reaction_rates<NR, R, NK>(c, Tr, R(1) / Tr, Yr, rho_phys, q);
+    reaction_rates<NR, R, NK>(c, Tr, inv_T, Yr, rho_phys, q);
     const R Fr = a.Floc ? ldg(a.Floc + r) : c.F;
     const R mur = c.nu_lat * powr<R>(Tr * c.T_ref_inv, c.mu_exp);
     // variable heat capacities: mixture c_p and the heat of each reaction at T_r
@@ -323,7 +332,7 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
     }
     // chemistry sources
     const R dt = c.dt_phys;
-    const R inv_rpF = R(1) / (rho_phys * Fr);
+    const R inv_rpF = recip(rho_phys * Fr);
     R qdot = R(0);
 #pragma unroll
     for (int j = 0; j < RMAX; ++j)
@@ -460,9 +469,9 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
       }
       R src;
       if (VCP && fi == 0) {
-        const R inv_cpr = R(1) / cp_r;
+        const R inv_cpr = recip(cp_r);
         dif = (dif + R(0.25) * Fr * mur * tflux) * gfac * inv_rho * inv_cpr;
-        src = (dt * qdot * inv_rpF + fd_dT * inv_rho / c.inv_cp) * inv_cpr;
+        src = (dt * qdot * inv_rpF + quot(fd_dT * inv_rho, c.inv_cp, recip(c.inv_cp))) * inv_cpr;
       } else if (fi == 0) {
         dif *= gfac * inv_rho;
         src = dt * qdot * inv_rpF * c.inv_cp + fd_dT * inv_rho;
@@ -478,7 +487,7 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
       const R pn = pr - adv + NA;
       if (fi == 0) {
         a.T_out[r] = pn;
-        lam += NA / Tr;
+        lam += quot(NA, Tr, inv_T);
         Tnew = pn;
       } else {
         a.Y_out[(size_t)(fi - 1) * N + r] = pn;
@@ -494,7 +503,8 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
     a.lam_out[r] = lam;
     if (c.closed) {
       // W_new / (R T_new rho_ref), pre-scaled; gas constant folded into I_scale
-      termI = c.I_scale / (sWn * Tnew);
+      const R wt = sWn * Tnew;
+      termI = quot(c.I_scale, wt, recip(wt));
       if (x == 0 && g.bc_lo[0] == BC_INLET) {
         const R rin = sizeof(R) == 4 ? (R)a.pth->rho_in : (R)a.pth->rho_in_d;
         termM += c.M_scale * rin * ldg(a.inlet_u + f);
@@ -512,7 +522,7 @@ __device__ __forceinline__ void fd_cell(const FDArgs<R>& a, int x, int y, int z,
 // warps per SM) and bound by issue at the largest; 6 species, step of chamber / flame, fields rolled at
 // 4 blocks / unrolled at 3: 256x1 (4 species) 9.5 / 8.5 us, 128x64 12.5 / 10.4, 512x128 14.6 / 12.5, 600x160 16.6 / 14.5,
 // 512x256 18.6 / 17.4, 1024x256 25.8 / 23.7, 2048x512 82.3 / 77.3; unrolled at 2 blocks 15.6 at 600x160, 24.9 at
-// 1024x256, 90.0 at 2048x512. In 3-D more fields in flight cost more registers than they hide (vessel
+// 1024x256, 90.0 at 2048x512 (with the reciprocals of recip: 1024x256 21.9, the small sizes as here). In 3-D more fields in flight cost more registers than they hide (vessel
 // 135x101x77: two per pass 124 us, rolled 117).
 constexpr int FD_UNROLLED = 3;
 template <int D, typename R, int NK, int NR, int VDEG = 0, bool MIX = false, int MINB = 4>
