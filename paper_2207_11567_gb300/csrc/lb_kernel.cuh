@@ -773,6 +773,16 @@ __device__ __forceinline__ void face_rules(const LBArgs<R>& a, int r, int x, int
   }
 }
 
+// With a wall list, its launch goes first and lets the launch over the other cells start beside it once the
+// kernels before both are complete (it waits for them before it triggers); the other cells read nothing it
+// writes. So that the launch after both finds both complete, the last block of the other cells waits for the
+// wall launch, and no other block does: it would hold its place on the SM until then. The list's few cells are
+// a chain of latencies (both launches, swirl burner with curved walls, one after the other / side by side:
+// 192x96x96 119 / 98.5 us, 384x192x192 638 / 625; with every block waiting 116.5).
+__device__ __forceinline__ void wall_wait(int n_wall) {
+  if (n_wall > 0 && blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) pdl_wait();
+}
+
 // WALLS = false: every fluid cell except those flagged LINK_WALL, one block row per (y, z).
 // WALLS = true: the flagged cells only, one thread per entry of the wall list, with the
 // interpolated bounce-back fix-up compiled in (so that it costs the other cells no registers).
@@ -782,6 +792,8 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
   const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz;
   int x, y, z, r, wrow = 0;
   if constexpr (WALLS) {
+    pdl_wait();
+    pdl_trigger();
     // one thread per cell of the interpolated-wall list (its position is the table row)
     wrow = blockIdx.x * LB_BLOCK + threadIdx.x;
     if (wrow >= a.n_wall) return;
@@ -790,6 +802,7 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
     y = (r / nx) % ny;
     z = r / (nx * ny);
   } else {
+    wall_wait(a.n_wall);
     // one block row of cells along x; y and z come from the grid (no integer division)
     x = blockIdx.x * blockDim.x + threadIdx.x;
     y = blockIdx.y;
@@ -872,8 +885,8 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
   }
   }
   // the thermodynamic-pressure state of this step: after the kernel that updates it (launched just
-  // before this one; the loads above read only what earlier kernels wrote)
-  pdl_wait();
+  // before this one; the loads above read only what earlier kernels wrote). With a wall list see wall_wait.
+  if (!WALLS && a.n_wall == 0) pdl_wait();
   if constexpr (THERMAL) {
     if constexpr (sizeof(R) == 8) lam += (R)a.pth->lb_lam_d;
     else lam += (R)a.pth->lb_lam;
@@ -1215,6 +1228,7 @@ __global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_IS
   constexpr uint32_t LINKS = (1u << Q) - 1u;
   const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz, N = a.geo.N;
   const int r = 2 * (blockIdx.x * LP_BLOCK + threadIdx.x);
+  wall_wait(a.n_wall);
   if (r >= N) return;
   const bool two = VEC || r + 1 < N;  // the last cell of an odd grid has no partner
   F2 rho = splat<F2>(1.0), lam = splat<F2>(0.0), T = splat<F2>(1.0);
@@ -1227,7 +1241,8 @@ __global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_IS
   // cells this launch updates: fluid ones, except those of the interpolated-wall list
   const bool act0 = (lw0 >> 30) == 2u, act1 = (lw1 >> 30) == 2u;
   if (!act0 && !act1) {
-    pdl_wait();  // an exit without it makes the thermal kernel slower (swirl 384x192x192: 575 us, so 563)
+    // an exit without it makes the thermal kernel slower (swirl 384x192x192: 575 us, so 563)
+    if (a.n_wall == 0) pdl_wait();
     return;
   }
   const int row = a.div_nx.div(r), z0 = D == 3 ? a.div_ny.div(row) : 0;
@@ -1262,7 +1277,7 @@ __global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_IS
         gz = splat<F2>(0.5) * (zp - zm);
       }
     }
-    pdl_wait();
+    if (a.n_wall == 0) pdl_wait();
 #pragma unroll
     for (int i = 0; i < Q; ++i) q[i] = pack2(cvt_pop<S, float>(raw0[i]), cvt_pop<S, float>(raw1[i]));
   } else {
@@ -1284,7 +1299,7 @@ __global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_IS
       gy = splat<F2>(0.5) * (pack2(rp[1], sp[1]) - pack2(rm[1], sm[1]));
       if constexpr (D == 3) gz = splat<F2>(0.5) * (pack2(rp[2], sp[2]) - pack2(rm[2], sm[2]));
     }
-    pdl_wait();
+    if (a.n_wall == 0) pdl_wait();
     float p0[Q], p1[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -1392,15 +1407,18 @@ cudaError_t launch_cells(const LBArgs<R>& a, cudaStream_t st, bool pdl) {
 }
 
 // pdl: the kernel may start while the one before it in the stream (the thermodynamic-pressure
-// update) runs; it reads that kernel's state after pdl_wait.
+// update) runs; it reads that kernel's state after pdl_wait. The wall list first (see wall_wait).
 template <int D, typename S, typename R>
 cudaError_t launch_lb(const LBArgs<R>& a, int thermal, int coll, cudaStream_t st, bool pdl) {
 #define LB_LAUNCH(TH, CO)                                                                         \
   do {                                                                                            \
-    cudaError_t e_ = launch_cells<D, S, R, TH, CO>(a, st, pdl);                                   \
+    if (a.n_wall > 0) {                                                                           \
+      cudaError_t e_ = launch_ex<LBArgs<R>>(lb_step_kernel<D, S, R, TH, CO, true>,                \
+                                            dim3((a.n_wall + LB_BLOCK - 1) / LB_BLOCK), dim3(LB_BLOCK), st, pdl, a); \
+      if (e_ != cudaSuccess) return e_;                                                           \
+    }                                                                                             \
+    cudaError_t e_ = launch_cells<D, S, R, TH, CO>(a, st, pdl || a.n_wall > 0);                   \
     if (e_ != cudaSuccess) return e_;                                                             \
-    if (a.n_wall > 0)                                                                             \
-      lb_step_kernel<D, S, R, TH, CO, true><<<(a.n_wall + LB_BLOCK - 1) / LB_BLOCK, LB_BLOCK, 0, st>>>(a); \
   } while (0)
   if (thermal) {
     if (coll == COLL_CUMULANT_FULL) LB_LAUNCH(true, COLL_CUMULANT_FULL);
