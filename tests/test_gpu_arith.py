@@ -1,0 +1,36 @@
+"""The kernels' own FP32 operations (reciprocal, quotient and root by Newton steps, the closure built on
+them) against CUDA's IEEE operators, bit for bit over all mantissas: tests/cuda/checks.cu, compiled here with
+the library's flags."""
+import ctypes as C
+import importlib.util
+import os
+import subprocess
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def build_checks(path):
+    """Compile tests/cuda/checks.cu into the folder ``path`` and load it."""
+    spec = importlib.util.spec_from_file_location("_hlbm_build", os.path.join(ROOT, "paper_2207_11567_gb300", "build.py"))
+    b = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(b)
+    so = os.path.join(str(path), "libchecks.so")
+    subprocess.run([b.nvcc(), *b.FLAGS, "-I", b.CSRC, "-shared", os.path.join(ROOT, "tests", "cuda", "checks.cu"),
+                    "-o", so], check=True)
+    return C.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def checks(tmp_path_factory):
+    lib = build_checks(tmp_path_factory.mktemp("checks"))
+    lib.check_tau.restype = C.c_longlong
+    lib.check_tau.argtypes = [C.c_float, C.c_float, C.c_int]
+    return lib
+
+
+@pytest.mark.parametrize("tau0, k, e", [(0.5, 0.736, -20), (0.5, 64.0, 10), (0.9, 0.25, -45)])
+def test_relaxation_time(checks, tau0, k, e):
+    assert checks.check_tau(tau0, k, e) == 0
