@@ -26,7 +26,8 @@ def build_checks(path):
 @pytest.fixture(scope="module")
 def checks(tmp_path_factory):
     lib = build_checks(tmp_path_factory.mktemp("checks"))
-    lib.check_tau.restype = C.c_longlong
+    for f in ("check_tau", "check_rcp", "check_sqrt", "check_div"):
+        getattr(lib, f).restype = C.c_longlong
     lib.check_tau.argtypes = [C.c_float, C.c_float, C.c_int]
     return lib
 
@@ -34,3 +35,20 @@ def checks(tmp_path_factory):
 @pytest.mark.parametrize("tau0, k, e", [(0.5, 0.736, -20), (0.5, 64.0, 10), (0.9, 0.25, -45)])
 def test_relaxation_time(checks, tau0, k, e):
     assert checks.check_tau(tau0, k, e) == 0
+
+
+@pytest.mark.parametrize("e", [-126, -67, -1, 63, 124])
+def test_reciprocal(checks, e):
+    """Exponents e and e + 1: 2^-126 .. 2^126."""
+    assert checks.check_rcp(e) == 0
+
+
+@pytest.mark.parametrize("e", [-67, -2, 1, 64, 126])
+def test_square_root(checks, e):
+    assert checks.check_sqrt(e) == 0
+
+
+def test_quotient(checks):
+    """2^24 random pairs; a numerator below 2^-100 may be off by one unit in the last place."""
+    assert checks.check_div(-100, 106, 0) == 0
+    assert checks.check_div(-105, -100, 1) == 0
