@@ -144,9 +144,9 @@ template <typename R> __device__ __forceinline__ R nu_of(const FDConst<R>& c, in
 }
 
 // Flame sensor: F_loc = 1 + (F - 1) tanh(beta Omega / Omega_0) with
-// Omega = max(Y_F, 0) max(Y_O, 0) exp(-T_s / T), a function of the cell's own state.
+// Omega = max(Y_F, 0) max(Y_O, 0) exp(-T_s / T), a function of the cell's own state (1 at T = 0).
 template <typename R> __device__ __forceinline__ R sensor_floc(const FDConst<R>& c, R T, R yf, R yo) {
-  const R om = fmax(yf, R(0)) * fmax(yo, R(0)) * exp(quot(-c.sensor_Ta, T, recip(T)));
+  const R om = fmax(yf, R(0)) * fmax(yo, R(0)) * exp(-c.sensor_Ta / T);
   return R(1) + (c.F - R(1)) * tanh(c.sensor_beta * om * c.inv_wref);
 }
 

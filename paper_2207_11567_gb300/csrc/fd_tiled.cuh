@@ -683,10 +683,7 @@ __global__ void __launch_bounds__(TT_THREADS, 2)
       }
     }
     if (active) {
-      if (a.Floc_out) {  // sensor_floc
-        const float om = fmaxf(yf_new, 0.0f) * fmaxf(yo_new, 0.0f) * expf(div_(-c.sensor_Ta, Tnew, rcp_(Tnew)));
-        a.Floc_out[r] = 1.0f + (c.F - 1.0f) * tanhf(c.sensor_beta * om * c.inv_wref);
-      }
+      if (a.Floc_out) a.Floc_out[r] = sensor_floc<float>(c, Tnew, yf_new, yo_new);
       a.rho_out[r] = rho;
       a.lam_out[r] = lam;
       if (c.closed) {

@@ -2,6 +2,7 @@
 // tests/test_gpu_arith.py with the library's flags. Each entry point returns how many of its values differ in
 // any bit from CUDA's IEEE operators, or -1 after a CUDA error.
 #include <cuda_runtime.h>
+#include "fd_kernel.cuh"
 #include "lb_kernel.cuh"
 
 using namespace hlbm;
@@ -57,6 +58,16 @@ __global__ void div_kernel(int ea_lo, int ea_hi, int off, unsigned long long* ba
   if (d < -off || d > off || signbit(q) != signbit(w)) atomicAdd(bad, 1ull);
 }
 
+// flame sensor at temperatures of a cell that holds no gas yet (0) or has blown up
+__global__ void sensor_kernel(const float* T, int n, float* out) {
+  FDConst<float> c{};
+  c.F = 8.0f;
+  c.sensor_Ta = 8400.0f;
+  c.sensor_beta = 10.0f;
+  c.inv_wref = 1e5f;
+  if ((int)threadIdx.x < n) out[threadIdx.x] = sensor_floc<float>(c, T[threadIdx.x], 0.04f, 0.2f);
+}
+
 constexpr int BLOCK = 256, MANTISSAS = 1 << 23;
 
 template <typename F> long long count(F launch) {
@@ -82,4 +93,9 @@ extern "C" long long check_sqrt(int e) {
 }
 extern "C" long long check_div(int ea_lo, int ea_hi, int off) {
   return count([=](unsigned long long* bad) { div_kernel<<<(1 << 24) / BLOCK, BLOCK>>>(ea_lo, ea_hi, off, bad); });
+}
+// F_loc at the n <= 32 temperatures T (device arrays)
+extern "C" int sensor(const float* T, int n, float* out) {
+  sensor_kernel<<<1, 32>>>(T, n, out);
+  return (int)cudaDeviceSynchronize();
 }

@@ -7,6 +7,7 @@ import os
 import subprocess
 
 import pytest
+import torch
 
 pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -52,3 +53,12 @@ def test_quotient(checks):
     """2^24 random pairs; a numerator below 2^-100 may be off by one unit in the last place."""
     assert checks.check_div(-100, 106, 0) == 0
     assert checks.check_div(-105, -100, 1) == 0
+
+
+def test_sensor_at_zero_temperature(checks):
+    """No reaction at T = 0 or without a finite exponent: F_loc = 1 (F = 8 here, reached when hot)."""
+    T = torch.tensor([0.0, 1e-30, 100.0, 2000.0], dtype=torch.float32, device="cuda")
+    out = torch.full_like(T, -1.0)
+    assert checks.sensor(C.c_void_p(T.data_ptr()), T.numel(), C.c_void_p(out.data_ptr())) == 0
+    assert out.tolist()[:3] == [1.0, 1.0, 1.0]
+    assert out[3].item() == 8.0
