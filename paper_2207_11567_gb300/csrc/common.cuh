@@ -211,6 +211,8 @@ template <typename R> struct LBArgs {
   const int* wall_cells;  // [n_wall] cells flagged LINK_WALL (interpolated bounce-back)
   const R* wall_q;        // [n_wall][Q] their wall fraction per pull direction (0.5: half-way)
   int n_wall;
+  int wall_planes;   // planes of blocks (lb_pair_kernel: blocks) in front that take the wall list
+  int pdl;           // lb_pair_kernel: the launch started beside the kernel before it (see pdl_wait)
   const R* rho;      // thermal: density at level n (lattice units)
   const R* lam;      // thermal: Lambda from the FD update (without the P_th term)
   const R* T;        // thermal: temperature at level n (viscosity law)

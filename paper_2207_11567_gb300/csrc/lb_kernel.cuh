@@ -780,43 +780,15 @@ __device__ __forceinline__ void face_rules(const LBArgs<R>& a, int r, int x, int
   }
 }
 
-// With a wall list, its launch goes first and lets the launch over the other cells start beside it once the
-// kernels before both are complete (it waits for them before it triggers); the other cells read nothing it
-// writes. So that the launch after both finds both complete, the last block of the other cells waits for the
-// wall launch, and no other block does: it would hold its place on the SM until then. The list's few cells are
-// a chain of latencies (both launches, swirl burner with curved walls, one after the other / side by side:
-// 192x96x96 119 / 98.5 us, 384x192x192 638 / 625; with every block waiting 116.5).
-__device__ __forceinline__ void wall_wait(int n_wall) {
-  if (n_wall > 0 && blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) pdl_wait();
-}
-
-// WALLS = false: every fluid cell except those flagged LINK_WALL, one block row per (y, z).
-// WALLS = true: the flagged cells only, one thread per entry of the wall list, with the
-// interpolated bounce-back fix-up compiled in (so that it costs the other cells no registers).
+// Update of the cell r = (x, y, z) by one thread.
+// WALLS = false: a fluid cell, unless flagged LINK_WALL.
+// WALLS = true: a flagged cell, row wrow of the wall table, with the interpolated bounce-back fix-up compiled
+// in (so that it costs the other cells no registers).
 template <int D, typename S, typename R, bool THERMAL, int COLL, bool WALLS>
-__global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const LBArgs<R> a) {
+__device__ __forceinline__ void lb_cell(const LBArgs<R>& a, const int x, const int y, const int z, const int r,
+                                        const int wrow) {
   constexpr int Q = Lat<D>::Q;
   const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz;
-  int x, y, z, r, wrow = 0;
-  if constexpr (WALLS) {
-    pdl_wait();
-    pdl_trigger();
-    // one thread per cell of the interpolated-wall list (its position is the table row)
-    wrow = blockIdx.x * LB_BLOCK + threadIdx.x;
-    if (wrow >= a.n_wall) return;
-    r = __ldg(a.wall_cells + wrow);
-    x = r % nx;
-    y = (r / nx) % ny;
-    z = r / (nx * ny);
-  } else {
-    wall_wait(a.n_wall);
-    // one block row of cells along x; y and z come from the grid (no integer division)
-    x = blockIdx.x * blockDim.x + threadIdx.x;
-    y = blockIdx.y;
-    z = blockIdx.z;
-    if (x >= nx) return;
-    r = x + nx * (y + ny * z);
-  }
   // the cell's rho, Lambda and T are loaded together with its link word (every cell has them)
   R rho = R(1), lam = R(0), T_early = R(0);
   if constexpr (THERMAL) {
@@ -826,7 +798,7 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
   }
   const uint32_t lw = __ldg(a.links + r);
   if (!(lw >> 31)) return;
-  if (!WALLS && (lw & LINK_WALL)) return;  // done by the wall-list launch
+  if (!WALLS && (lw & LINK_WALL)) return;  // done by the blocks of the wall list
   const size_t N = (size_t)a.geo.N;
   const S* __restrict__ gin = (const S*)a.g_in;
   const R third = R(1) / R(3);
@@ -892,8 +864,8 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
   }
   }
   // the thermodynamic-pressure state of this step: after the kernel that updates it (launched just
-  // before this one; the loads above read only what earlier kernels wrote). With a wall list see wall_wait.
-  if (!WALLS && a.n_wall == 0) pdl_wait();
+  // before this one; the loads above read only what earlier kernels wrote)
+  pdl_wait();
   if constexpr (THERMAL) {
     if constexpr (sizeof(R) == 8) lam += (R)a.pth->lb_lam_d;
     else lam += (R)a.pth->lb_lam;
@@ -1178,6 +1150,33 @@ __global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const 
   if (!isfinite(usq)) atomicOr(a.flag, 1);
 }
 
+// Cell i of the wall list, one thread each.
+template <int D, typename S, typename R, bool THERMAL, int COLL>
+__device__ __forceinline__ void lb_wall_cell(const LBArgs<R>& a, const int i) {
+  if (i >= a.n_wall) return;
+  const int nx = a.geo.nx, ny = a.geo.ny, r = __ldg(a.wall_cells + i);
+  lb_cell<D, S, R, THERMAL, COLL, true>(a, r % nx, (r / nx) % ny, r / (nx * ny), r, i);
+}
+
+// One thread per cell, one block row of cells along x; y and z come from the grid (no integer division).
+// LIST: the first planes of blocks (wall_planes) take the wall list, the others the cells that are not on
+// it. In one launch the list's few cells, a chain of latencies, run beside the others and need no wait of
+// their own (see launch_lb).
+template <int D, typename S, typename R, bool THERMAL, int COLL, bool LIST>
+__global__ void __launch_bounds__(LB_BLOCK, LB_MIN_BLOCKS) lb_step_kernel(const LBArgs<R> a) {
+  int z = blockIdx.z;
+  if constexpr (LIST) {
+    if (z < a.wall_planes) {
+      lb_wall_cell<D, S, R, THERMAL, COLL>(
+          a, (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * z)) * blockDim.x + threadIdx.x);
+      return;
+    }
+    z -= a.wall_planes;
+  }
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  if (x >= a.geo.nx) return;
+  lb_cell<D, S, R, THERMAL, COLL, false>(a, x, y, z, x + a.geo.nx * (y + a.geo.ny * z), 0);
+}
 
 // ------------------------------------------------------------------ two cells per thread
 // Stream-collide of FP32 arithmetic with full relaxation of the orders 3..6 (the default rates): a
@@ -1229,13 +1228,23 @@ template <bool VEC> __device__ __forceinline__ F2 ld_pair(const float* p, bool t
   return pack2(__ldg(p), __ldg(p + (two ? 1 : 0)));
 }
 
-template <int D, typename S, bool THERMAL, bool VEC>
+// LIST: the first blocks (wall_planes of them) take the wall list, one cell per thread, as in lb_step_kernel.
+// a.pdl: a wait that every launch executes costs the others 1% (cold swirl 256x128x128 2875 against 2844 us
+// per 20 steps, vessel 135x101x77 1568 against 1560 per 10).
+template <int D, typename S, bool THERMAL, bool VEC, bool LIST>
 __global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_ISOTHERMAL) lb_pair_kernel(const LBArgs<float> a) {
   constexpr int Q = Lat<D>::Q;
   constexpr uint32_t LINKS = (1u << Q) - 1u;
   const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz, N = a.geo.N;
-  const int r = 2 * (blockIdx.x * LP_BLOCK + threadIdx.x);
-  wall_wait(a.n_wall);
+  int block = blockIdx.x;
+  if constexpr (LIST) {
+    if (block < a.wall_planes) {
+      lb_wall_cell<D, S, float, THERMAL, COLL_CUMULANT_FULL>(a, block * LP_BLOCK + threadIdx.x);
+      return;
+    }
+    block -= a.wall_planes;
+  }
+  const int r = 2 * (block * LP_BLOCK + threadIdx.x);
   if (r >= N) return;
   const bool two = VEC || r + 1 < N;  // the last cell of an odd grid has no partner
   F2 rho = splat<F2>(1.0), lam = splat<F2>(0.0), T = splat<F2>(1.0);
@@ -1249,7 +1258,7 @@ __global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_IS
   const bool act0 = (lw0 >> 30) == 2u, act1 = (lw1 >> 30) == 2u;
   if (!act0 && !act1) {
     // an exit without it makes the thermal kernel slower (swirl 384x192x192: 575 us, so 563)
-    if (a.n_wall == 0) pdl_wait();
+    if (THERMAL && a.pdl) pdl_wait();
     return;
   }
   const int row = a.div_nx.div(r), z0 = D == 3 ? a.div_ny.div(row) : 0;
@@ -1284,7 +1293,7 @@ __global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_IS
         gz = splat<F2>(0.5) * (zp - zm);
       }
     }
-    if (a.n_wall == 0) pdl_wait();
+    if (THERMAL && a.pdl) pdl_wait();
 #pragma unroll
     for (int i = 0; i < Q; ++i) q[i] = pack2(cvt_pop<S, float>(raw0[i]), cvt_pop<S, float>(raw1[i]));
   } else {
@@ -1306,7 +1315,7 @@ __global__ void __launch_bounds__(LP_BLOCK, THERMAL ? LP_MIN_THERMAL : LP_MIN_IS
       gy = splat<F2>(0.5) * (pack2(rp[1], sp[1]) - pack2(rm[1], sm[1]));
       if constexpr (D == 3) gz = splat<F2>(0.5) * (pack2(rp[2], sp[2]) - pack2(rm[2], sm[2]));
     }
-    if (a.n_wall == 0) pdl_wait();
+    if (THERMAL && a.pdl) pdl_wait();
     float p0[Q], p1[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -1381,52 +1390,64 @@ template <typename S> bool pair_aligned(const LBArgs<float>& a, bool thermal) {
   return a.geo.nx % 2 == 0 && f % 8 == 0 && ((uintptr_t)a.g_in | (uintptr_t)a.g_out) % (2 * sizeof(S)) == 0;
 }
 
-template <int D, typename S, bool THERMAL>
+template <int D, typename S, bool THERMAL, bool LIST>
 cudaError_t launch_pair(LBArgs<float> a, cudaStream_t st, bool pdl) {
   a.div_nx = FastDiv((uint32_t)a.geo.nx);
   a.div_ny = FastDiv((uint32_t)a.geo.ny);
+  a.wall_planes = LIST ? (a.n_wall + LP_BLOCK - 1) / LP_BLOCK : 0;
+  a.pdl = pdl;
   const int pairs = (a.geo.N + 1) / 2;
-  const dim3 grid((pairs + LP_BLOCK - 1) / LP_BLOCK);
+  const dim3 grid(a.wall_planes + (pairs + LP_BLOCK - 1) / LP_BLOCK);
   if (pair_aligned<S>(a, THERMAL))
-    return launch_ex<LBArgs<float>>(lb_pair_kernel<D, S, THERMAL, true>, grid, dim3(LP_BLOCK), st, pdl, a);
-  return launch_ex<LBArgs<float>>(lb_pair_kernel<D, S, THERMAL, false>, grid, dim3(LP_BLOCK), st, pdl, a);
+    return launch_ex<LBArgs<float>>(lb_pair_kernel<D, S, THERMAL, true, LIST>, grid, dim3(LP_BLOCK), st, pdl, a);
+  return launch_ex<LBArgs<float>>(lb_pair_kernel<D, S, THERMAL, false, LIST>, grid, dim3(LP_BLOCK), st, pdl, a);
 }
 
-// The stream-collide of every cell not on the wall list. FP32 arithmetic at the default rates: two cells
-// per thread in 3-D, and in 2-D from PAIR_MIN_2D cells on; below that the grid does not fill the GPU
+// FP32 arithmetic at the default rates: two cells per thread in 3-D, and in 2-D from PAIR_MIN_2D cells on; below that the grid does not fill the GPU
 // with pairs and the longer threads cost what the fewer instructions save (chamber step, one cell / two:
 // 256x64 13.47 / 13.53 us, 512x128 14.48 / 14.48, 600x200 17.58 / 16.59, 1024x256 27.20 / 25.07; 3-D
 // gains at every size, e.g. periodic box of 82,615 cells 10.35 / 5.47 us). Otherwise one cell per thread.
 constexpr int PAIR_MIN_2D = 100000;
-template <int D, typename S, typename R, bool THERMAL, int COLL>
-cudaError_t launch_cells(const LBArgs<R>& a, cudaStream_t st, bool pdl) {
+template <int D, typename S, typename R, bool THERMAL, int COLL, bool LIST>
+cudaError_t launch_cells(LBArgs<R> a, cudaStream_t st, bool pdl) {
   constexpr bool PAIR = COLL == COLL_CUMULANT_FULL && sizeof(R) == 4;
   if constexpr (PAIR) {
-    if (D == 3 || a.geo.N >= PAIR_MIN_2D) return launch_pair<D, S, THERMAL>(a, st, pdl);
+    if (D == 3 || a.geo.N >= PAIR_MIN_2D) return launch_pair<D, S, THERMAL, LIST>(a, st, pdl);
   }
   if constexpr (!PAIR || D == 2) {
     // blocks of one warp where larger ones would leave SMs empty (planar flame 256x8 FP64, with the FD
     // update spread the same way: 122 -> 34 us per step)
     const int block = a.geo.N < 32768 ? 32 : LB_BLOCK;
-    const dim3 grid((a.geo.nx + block - 1) / block, a.geo.ny, a.geo.nz);
-    return launch_ex<LBArgs<R>>(lb_step_kernel<D, S, R, THERMAL, COLL, false>, grid, dim3(block), st, pdl, a);
+    dim3 grid((a.geo.nx + block - 1) / block, a.geo.ny, a.geo.nz);
+    const auto kernel = lb_step_kernel<D, S, R, THERMAL, COLL, LIST>;
+    a.wall_planes = 0;
+    if constexpr (LIST) {
+      const size_t plane = (size_t)block * grid.x * grid.y;
+      a.wall_planes = (int)((a.n_wall + plane - 1) / plane);
+      if (grid.z + a.wall_planes > 65535u) {  // no planes left for the list: a launch of its own
+        a.wall_planes = 1;
+        const cudaError_t e = launch_ex<LBArgs<R>>(kernel, dim3((a.n_wall + block - 1) / block), dim3(block), st, pdl, a);
+        if (e != cudaSuccess) return e;
+        a.wall_planes = 0;
+        pdl = false;
+      }
+      grid.z += a.wall_planes;
+    }
+    return launch_ex<LBArgs<R>>(kernel, grid, dim3(block), st, pdl, a);
   }
 }
 
 // pdl: the kernel may start while the one before it in the stream (the thermodynamic-pressure
-// update) runs; it reads that kernel's state after pdl_wait. The wall list first (see wall_wait).
+// update) runs; it reads that kernel's state after pdl_wait. The cells of a wall list, a chain of latencies,
+// take the first blocks of the same launch. As a launch of their own just before, that the other cells'
+// started beside, the two needed a wait for each other; on a second stream, forked and joined by events, a
+// graph ran them one after the other. Step of the swirl burner with curved walls, launch of its own beside /
+// second stream / same launch: 96x48x48 62.4 / 64.1 / 53.0 us, 192x96x96 250 / 263 / 248; cold 128x64x64 FP32
+// 53.0 / 48.5 / 45.4, FP16 27.9 / 33.7 / 22.8.
 template <int D, typename S, typename R>
 cudaError_t launch_lb(const LBArgs<R>& a, int thermal, int coll, cudaStream_t st, bool pdl) {
-#define LB_LAUNCH(TH, CO)                                                                         \
-  do {                                                                                            \
-    if (a.n_wall > 0) {                                                                           \
-      cudaError_t e_ = launch_ex<LBArgs<R>>(lb_step_kernel<D, S, R, TH, CO, true>,                \
-                                            dim3((a.n_wall + LB_BLOCK - 1) / LB_BLOCK), dim3(LB_BLOCK), st, pdl, a); \
-      if (e_ != cudaSuccess) return e_;                                                           \
-    }                                                                                             \
-    cudaError_t e_ = launch_cells<D, S, R, TH, CO>(a, st, pdl || a.n_wall > 0);                   \
-    if (e_ != cudaSuccess) return e_;                                                             \
-  } while (0)
+#define LB_LAUNCH(TH, CO) \
+  return a.n_wall > 0 ? launch_cells<D, S, R, TH, CO, true>(a, st, pdl) : launch_cells<D, S, R, TH, CO, false>(a, st, pdl)
   if (thermal) {
     if (coll == COLL_CUMULANT_FULL) LB_LAUNCH(true, COLL_CUMULANT_FULL);
     else if (coll == COLL_CUMULANT) LB_LAUNCH(true, COLL_CUMULANT);
@@ -1437,7 +1458,6 @@ cudaError_t launch_lb(const LBArgs<R>& a, int thermal, int coll, cudaStream_t st
     else LB_LAUNCH(false, COLL_BGK);
   }
 #undef LB_LAUNCH
-  return cudaGetLastError();
 }
 
 }  // namespace hlbm
