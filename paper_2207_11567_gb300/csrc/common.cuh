@@ -136,8 +136,10 @@ template <> __device__ __forceinline__ void st_pop<__half, float>(__half* p, flo
 // Programmatic dependent launch: a kernel launched with programmatic stream serialization may
 // start before its predecessor in the stream has finished. pdl_wait blocks until that predecessor
 // has completed and its writes are visible (it returns at once without one); pdl_trigger lets the
-// next such kernel start. Kernels call pdl_trigger only after pdl_wait, so that when a kernel
-// starts, every kernel before its predecessor has completed.
+// next such kernel start. Every kernel that calls pdl_trigger has called pdl_wait before it, so that when a
+// kernel starts, every kernel before its predecessor has completed and what that one left is visible; what
+// the predecessor itself writes is read only after pdl_wait. Every block that goes on past its first test of
+// the cell executes pdl_wait once, at its end if it reads nothing of the predecessor's (fd_tiled_kernel).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -538,7 +538,8 @@ __global__ void __launch_bounds__(FD_BLOCK, sizeof(R) == 4 ? MINB : 1)
   bool inside;
   if (a.wall_list) {
     // the tiled update of the other cells may start: it writes none of what this launch reads, and what both
-    // read is complete (this launch waited for its predecessors before its first block)
+    // read is complete behind this wait (at once in the ordinary launch that this is)
+    pdl_wait();
     pdl_trigger();
     // one thread per listed cell (a 1-D grid of blocks of the same shape)
     const int wrow = blockIdx.x * FD_BLOCK + threadIdx.x + FDShape<D>::X * (threadIdx.y + FDShape<D>::Y * threadIdx.z);
