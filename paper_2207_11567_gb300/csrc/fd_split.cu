@@ -8,11 +8,14 @@
 // the rate law are independent tasks, dealt out to the warps and passed through shared memory; then
 // each warp does the faces, diffusion and sources of its own field. Formulas as in fd_cell, with the
 // shared reciprocals formed once per cell.
-// Measured on 256x8 cells, 4 species, one reaction: FD + stream-collide 122 -> 34 us per step (FD update
-// 113 us in 8 blocks of fd_step_kernel).
-// Taken up to FD_SPLIT_MAX cells: there the warps of one field per cell still fit the GPU's
-// sub-partitions about once or twice; above, fd_step_kernel fills the GPU without the shared
-// quantities being formed by every warp.
+// Measured on 256x8 cells, 4 species, one reaction, one run alone: FD + stream-collide 122 -> 34 us per step
+// (FD update 113 us in 8 blocks of fd_step_kernel).
+// Taken up to FD_SPLIT_MAX cells, six blocks per SM: with a seventh on some of them the warps, which all form
+// the shared quantities, cost more than fd_step_kernel's blocks of 256 cells with every SM busy. Whole step,
+// fd_step_kernel / this: 6 species (2 reactions) 16,384 cells 156.7 / 101.5 us, 24,576 161.8 / 148.4, 29,184
+// 161.8 / 151.6, 30,208 164.5 / 187.3, 32,768 166.2 / 193.1; 4 species (1 reaction) 16,384 116.9 / 74.8,
+// 24,576 121.9 / 120.7, 29,184 122.0 / 122.1, 32,768 126.0 / 128.3; 8 species 28,672 185.8 / 175.7, 32,768
+// 190.4 / 206.2.
 #include "fd_kernel.cuh"
 #include "launch.h"
 

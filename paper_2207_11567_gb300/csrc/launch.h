@@ -28,7 +28,7 @@ cudaError_t fd_tiled_set_mask(FDTiledMaps& m, const Geo& g, const uint8_t* mask,
 cudaError_t launch_fd_tiled(const FDArgs<float>& a, const FDTiledMaps& m, int cur, cudaStream_t st, bool pdl);
 
 // fd_split.cu: FD update of small 2-D FP64 grids, one warp per field (no options, no wall weights)
-constexpr int FD_SPLIT_MAX = 32768;
+constexpr int FD_SPLIT_MAX = 6 * 152 * 32;  // 6 blocks of 32 cells per SM (fd_split.cu)
 int fd_split_blocks(const Geo& g);
 cudaError_t launch_fd_split(const FDArgs<double>& a, cudaStream_t st);
 
