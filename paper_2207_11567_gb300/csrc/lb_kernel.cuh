@@ -1403,6 +1403,22 @@ cudaError_t launch_pair(LBArgs<float> a, cudaStream_t st, bool pdl) {
   return launch_ex<LBArgs<float>>(lb_pair_kernel<D, S, THERMAL, false, LIST>, grid, dim3(LP_BLOCK), st, pdl, a);
 }
 
+// Small FP64 grids run blocks of one warp where the most loaded SM then holds fewer of the warps with cells:
+// an FP64 instruction holds its sub-partition for 32 clocks, so the step lasts as long as the SM with the most
+// warps. Blocks of 128 / of 32: planar flame 256x8 34.4 / 33.8 us per step, 2-D boxes 200x80 10.3 / 7.2,
+// 129x240 17.4 / 10.3, level at 33x400 (8.2) and 97x300 (10.3; BGK 13.7 / 14.4, which the rule leaves at 128),
+// 3-D 129x14x14 38.9 / 25.6. In 3-D only where a row takes several blocks of 128: with shorter rows the one-warp
+// blocks of a row's full and last warps fall on the sub-partitions unevenly (33x28x28 27.4 / 36.7, 36x29x29
+// 33.8 / 39.0). FP32 is bound by latency and gains nothing (2-D box 33x900 4.1 / 5.1).
+constexpr int LB_ONE_WARP_MAX = 32768, LB_SMS = 152;
+template <int D, typename R> bool one_warp_blocks(const Geo& g) {
+  if (sizeof(R) == 4 || g.N >= LB_ONE_WARP_MAX || (D == 3 && g.nx <= LB_BLOCK)) return false;
+  const long long rows = (long long)g.ny * g.nz, blocks = rows * ((g.nx + LB_BLOCK - 1) / LB_BLOCK);
+  const long long warps = rows * ((g.nx + 31) / 32);
+  // warps per SM: ceil(warps / SMs) against ceil(blocks / SMs) of warps / blocks each
+  return (warps + LB_SMS - 1) / LB_SMS * blocks < (blocks + LB_SMS - 1) / LB_SMS * warps;
+}
+
 // FP32 arithmetic at the default rates: two cells per thread in 3-D, and in 2-D from PAIR_MIN_2D cells on; below that the grid does not fill the GPU
 // with pairs and the longer threads cost what the fewer instructions save (chamber step, one cell / two:
 // 256x64 13.47 / 13.53 us, 512x128 14.48 / 14.48, 600x200 17.58 / 16.59, 1024x256 27.20 / 25.07; 3-D
@@ -1415,9 +1431,7 @@ cudaError_t launch_cells(LBArgs<R> a, cudaStream_t st, bool pdl) {
     if (D == 3 || a.geo.N >= PAIR_MIN_2D) return launch_pair<D, S, THERMAL, LIST>(a, st, pdl);
   }
   if constexpr (!PAIR || D == 2) {
-    // blocks of one warp where larger ones would leave SMs empty (planar flame 256x8 FP64, with the FD
-    // update spread the same way: 122 -> 34 us per step)
-    const int block = a.geo.N < 32768 ? 32 : LB_BLOCK;
+    const int block = one_warp_blocks<D, R>(a.geo) ? 32 : LB_BLOCK;
     dim3 grid((a.geo.nx + block - 1) / block, a.geo.ny, a.geo.nz);
     const auto kernel = lb_step_kernel<D, S, R, THERMAL, COLL, LIST>;
     a.wall_planes = 0;
