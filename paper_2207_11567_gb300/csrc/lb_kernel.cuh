@@ -783,9 +783,10 @@ __device__ __forceinline__ void face_rules(const LBArgs<R>& a, int r, int x, int
 // Update of the cell r = (x, y, z) by one thread.
 // WALLS = false: a fluid cell, unless flagged LINK_WALL.
 // WALLS = true: a flagged cell, row wrow of the wall table, with the interpolated bounce-back fix-up compiled
-// in (so that it costs the other cells no registers).
+// in (so that it costs the other cells no registers). The arguments come by value, as a kernel's do: by
+// reference nvcc fused other products of the inlet and outlet rules (a last place in a few cells).
 template <int D, typename S, typename R, bool THERMAL, int COLL, bool WALLS>
-__device__ __forceinline__ void lb_cell(const LBArgs<R>& a, const int x, const int y, const int z, const int r,
+__device__ __forceinline__ void lb_cell(const LBArgs<R> a, const int x, const int y, const int z, const int r,
                                         const int wrow) {
   constexpr int Q = Lat<D>::Q;
   const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz;
