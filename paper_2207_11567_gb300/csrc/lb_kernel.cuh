@@ -611,9 +611,10 @@ __device__ __forceinline__ void collide_central(F2* q, LBCell<3, F2, true>& c, c
     const V n2 = fma_(two, o2, fma_(e2, e2, fma_(e0, e0, e1 * e1)));
     tau = smag_tau(tau0, n2, splat<V>(a.smag_k));
   }
-  const V o1 = one - rcp_(tau), obt = splat<V>(1.0f - a.omega_b) * tr;
+  const V o1 = one - rcp_(tau), ob = splat<V>(1.0f - a.omega_b);
   // ---- relaxed second-order moments and the higher ones without cumulants
-  const V sxx = fma_(o1, q[2] - tr, obt), syy = fma_(o1, q[6] - tr, obt), szz = fma_(o1, q[18] - tr, obt);
+  const V sxx = fma_(ob, tr, mul_rn(o1, q[2] - tr)), syy = fma_(ob, tr, mul_rn(o1, q[6] - tr));
+  const V szz = fma_(ob, tr, mul_rn(o1, q[18] - tr));
   const V sxy = mul_rn(o1, q[4]), sxz = mul_rn(o1, q[10]), syz = mul_rn(o1, q[12]);
   const V tx = third + sxx, ty = third + syy, tz = third + szz;
   const V s2xy = two * sxy, s2xz = two * sxz, sxxyy = mul_rn(sxx, syy);

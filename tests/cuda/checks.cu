@@ -99,3 +99,49 @@ extern "C" int sensor(const float* T, int n, float* out) {
   sensor_kernel<<<1, 32>>>(T, n, out);
   return (int)cudaDeviceSynchronize();
 }
+
+// One thermal D3Q27 stream-collide at the default rates with one thread per cell (two = 0) or two cells per
+// thread (two = 1), populations of FP16 (half = 1) or FP32; bc: low and high code of x, y, z; device arrays.
+__device__ PthState g_pth;
+__device__ int g_flag;
+
+template <typename S> cudaError_t stream_collide_of(int two, const LBArgs<float>& a) {
+  if (two) return launch_pair<3, S, true, false>(a, 0, false);
+  const dim3 grid((a.geo.nx + LB_BLOCK - 1) / LB_BLOCK, a.geo.ny, a.geo.nz);
+  return launch_ex<LBArgs<float>>(lb_step_kernel<3, S, float, true, COLL_CUMULANT_FULL, false>, grid, dim3(LB_BLOCK), 0, false, a);
+}
+
+extern "C" int stream_collide(int two, int half, const int* n, const int* bc, const void* g_in, const unsigned int* links,
+                              const float* rho, const float* lam, const float* T, const float* inlet, const float* u_in,
+                              float lb_lam, float omega_b, float smag_k, float P_ref, void* g_out, float* u_out,
+                              float* ph) {
+  LBArgs<float> a{};
+  a.geo = Geo{n[0], n[1], n[2], n[0] * n[1] * n[2], {bc[0], bc[2], bc[4]}, {bc[1], bc[3], bc[5]}};
+  PthState p{};
+  p.lb_lam = lb_lam;
+  if (cudaMemcpyToSymbol(g_pth, &p, sizeof(p)) != cudaSuccess) return -1;
+  void *pth = nullptr, *flag = nullptr;
+  if (cudaGetSymbolAddress(&pth, g_pth) != cudaSuccess || cudaGetSymbolAddress(&flag, g_flag) != cudaSuccess) return -1;
+  a.g_in = g_in;
+  a.g_out = g_out;
+  a.links = links;
+  a.rho = rho;
+  a.lam = lam;
+  a.T = T;
+  a.inlet_u = inlet;
+  a.u_in = u_in;
+  a.u = u_out;
+  a.write_u = 1;
+  a.ph_out = ph;
+  a.pth = (const PthState*)pth;
+  a.flag = (int*)flag;
+  a.nu_lat = 0.002f;
+  a.T_ref_inv = 1.0f / 300.0f;
+  a.mu_exp = 0.7f;
+  a.smag_k = smag_k;
+  a.P_ref = P_ref;
+  a.omega_b = omega_b;
+  a.om3 = a.om4 = a.om5 = a.om6 = 1.0f;
+  const cudaError_t e = half ? stream_collide_of<__half>(two, a) : stream_collide_of<float>(two, a);
+  return e != cudaSuccess ? (int)e : (int)cudaDeviceSynchronize();
+}
