@@ -61,3 +61,18 @@ def test_grid_without_planes_to_spare():
     for deep, flat in zip(run(65535), run(4)):
         assert np.isfinite(flat).all() and np.abs(flat).max() > 0
         assert (deep == flat[:, :1]).all()
+
+
+def test_curved_walls_f16():
+    """FP16 storage against the FP64 oracle: relative L2 of u, as in the other FP16 tests."""
+    from oracle.step import Oracle
+    from tests.parity import compare, gpu_run, rel_l2
+    wl = W.generate.swirl_3d(40, 20, 20, curved=True, storage="f16", seed=4)
+    c, d, q = wl.info["wall_links"]
+    q = np.asarray(q, dtype=np.float32).astype(np.float64)
+    wl.info["wall_links"] = (c, d, q)
+    dense = np.zeros((27, wl.N))
+    dense[d, c] = q
+    o = Oracle(wl.cfg, wl.mask, wl.inlet_u, qwall=dense)
+    st = o.run(o.round_state(o.init_state(T=wl.T, Y=wl.Y, u=wl.u, P_h=wl.P_h, g_pert=wl.g_pert)), 20)
+    assert compare(wl, gpu_run(wl, 20), st, metric=rel_l2)["u"] <= 2e-3
