@@ -191,7 +191,8 @@ constexpr int LB_BLOCK = 128;
 constexpr uint32_t LINK_WALL = 1u << 30;
 
 // Quotient of a 31-bit unsigned number by a divisor known at launch: one high product, one add,
-// one shift (multiplier 2^32 (2^s - d) / d + 1 with s = ceil(log2 d)).
+// one shift (the round-up multiplier 2^32 (2^s - d) / d + 1 with s = ceil(log2 d) of Granlund and Montgomery,
+// "Division by invariant integers using multiplication", 1994).
 struct FastDiv {
   uint32_t mul = 1, shift = 0;
   FastDiv() = default;

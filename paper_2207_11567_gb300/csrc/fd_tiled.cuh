@@ -31,7 +31,7 @@
 //   a tile that holds fluid, and a row of cells without a fluid face skips the face work.
 //
 // Bound by instruction issue (58% of the issue slots, the rest waits on barriers, shared memory and the
-// chain of each face), not by memory: swirl burner 384x192x192, FP32, 10.97 M fluid cells, 808 us per
+// chain of each face), not by memory: swirl burner 384x192x192, FP32, 11.08 M fluid cells, 808 us per
 // update with one field per instruction and all tiles, 698 us so (126 us of traffic at the copy rate).
 // Packed faces, reciprocals and conversions: 808 -> 765 us; rows without fluid 759; tile list 698.
 //
