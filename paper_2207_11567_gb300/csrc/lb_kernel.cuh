@@ -437,7 +437,7 @@ __device__ __forceinline__ void collide_full(V* q, LBCell<D, V, THERMAL>& c, con
 // ------------------------------------------------------------ collision of two cells, D3Q27 thermal
 // The update of collide_full with central moments (axis-by-axis transform of all of them), operation by operation
 // in the arithmetic of the one-cell kernel's FP32 form: same order, same products fused into an add,
-// so that its results are the same bits. Why here: a reacting flow turns rounding into differences
+// so that its results are the same bits (tests/test_gpu_pair_bits.py). Why here: a reacting flow turns rounding into differences
 // of another size (a fuel fraction of order 1/2 crossing zero, a face velocity changing sign: 1e-8 in u
 // becomes 1e-3 of the pressure fluctuation in 20 steps), so the arithmetic of reacting 3-D runs does not
 // change with the kernel that carries it.
